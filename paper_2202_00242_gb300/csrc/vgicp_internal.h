@@ -18,9 +18,12 @@ constexpr int kMaxDevices = 64;
 // ---- error reporting -------------------------------------------------------
 int set_error(int code, const std::string& msg);
 int check_cuda(cudaError_t e, const char* what);  // cudaErrorMemoryAllocation -> OOM
-// Every device allocation of the library (cudaMalloc, or cudaMallocAsync on st
-// when stream_ordered); fails without allocating while the test hook asks.
+// Every device allocation of the library (cudaMalloc, or stream-ordered on st from
+// the library's scratch pool); fails without allocating while the test hook asks.
 cudaError_t device_malloc(void** p, size_t bytes, cudaStream_t st, bool stream_ordered);
+// Maps and plans alive (n = 1 or -1): with the last one the scratch pools give
+// their memory back.
+void count_owners(int n);
 #define VGICP_CUDA_TRY(call)                                   \
   do {                                                         \
     cudaError_t e__ = (call);                                  \

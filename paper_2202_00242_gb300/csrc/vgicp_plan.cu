@@ -218,6 +218,7 @@ void destroy_plan(vgicp_plan* P) {
   if (P->cap) cudaStreamDestroy(P->cap);
   if (P->d_block) cudaFree(P->d_block);
   delete P;
+  count_owners(-1);
 }
 
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
@@ -245,6 +246,7 @@ int vgicp_plan_create(vgicp_map* const* maps, int32_t n_maps, const vgicp_cloud*
   if (opts && opts->tile > 0 && opts->tile < kMinItem)
     return set_error(VGICP_ERR_INVALID_ARG, "plan item size must be at least 2048 points");
   vgicp_plan* P = new vgicp_plan();
+  count_owners(1);
   cudaGetDevice(&P->device);
   P->n_pairs = (int32_t)n_pairs;
   P->neighbours = neighbours;
