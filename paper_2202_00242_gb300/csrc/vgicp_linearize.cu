@@ -213,8 +213,9 @@ __device__ __forceinline__ void add_term_t(float* acc, const float* R, float x, 
   const float i22 = fmaf(m00, m11, -m01 * m01);
   const float det = fmaf(m00, i00, fmaf(m01, i01, m02 * i02));
   const float s = rcp_approx(det);
-  const float w00 = i00 * s, w01 = i01 * s, w02 = i02 * s;
-  const float w11 = i11 * s, w12 = i12 * s, w22 = i22 * s;
+  // (rounded before they are added below, so that every kernel forms the same sums)
+  const float w00 = __fmul_rn(i00, s), w01 = __fmul_rn(i01, s), w02 = __fmul_rn(i02, s);
+  const float w11 = __fmul_rn(i11, s), w12 = __fmul_rn(i12, s), w22 = __fmul_rn(i22, s);
   // u = W' d'
   const float u0 = fmaf(w00, d0, fmaf(w01, d1, w02 * d2));
   const float u1 = fmaf(w01, d0, fmaf(w11, d1, w12 * d2));
@@ -1141,6 +1142,330 @@ __global__ void __launch_bounds__(kThreads, VGICP_COMPACT_MIN_BLOCKS)
 }  // namespace compact
 
 
+// ---------------------------------------------------------------------------
+// Few long work items (1 neighbour): one cluster of 8 CTAs per item.
+//
+// A thread of the per-point kernel takes its points of an item one after the other
+// (64 of a 16K item), and a factor set of a few items, a sliding window for
+// instance, lasts as long as that chain: 72 us for ten factors of 20,000 points on
+// 20 of 152 SMs.  Here CTA w of the cluster takes what warp w of the per-point
+// kernel takes.  Its 8 warps look up and invert 16 points of every lane at once (two
+// per thread, in flight together) and leave them in shared memory; then each
+// accumulator is summed over them by one thread per lane, in the order in which the
+// per-point kernel adds them, so every sum is the same bit for bit.  The
+// accumulators are dealt to warps 0 - 4; the CTAs' sums meet in the first CTA
+// through distributed shared memory.
+//
+// The SMs do more work per point this way (all threads wait for the sums), so it
+// is for few items (split_items).  Bounded by the latency of a round (two loads, a
+// barrier) and by the sums' shared-memory reads.
+// ---------------------------------------------------------------------------
+namespace split {
+constexpr int kCtas = 8;          // CTAs per item = warps of the per-point kernel
+constexpr int kWarps = 8;
+constexpr int kThreads = 32 * kWarps;
+constexpr int kPer = 2;           // points per thread and round
+constexpr int kRound = kWarps * kPer;
+static_assert(kCtas * 32 == kSimpleThreads, "one CTA per warp of the per-point kernel");
+
+// What the sums need of a point: MODE 0: adj(M') (6), 1 / det, u (3), d (3), x, y,
+// z; modes 1 - 3: u, d, x, y, z and C_k u.
+__host__ __device__ constexpr int values(int mode) { return mode == 0 ? 16 : mode == 3 ? 12 : mode == 2 ? 9 : 6; }
+
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::
+                   : "memory");
+}
+// Address of a shared-memory object of CTA `rank` of the cluster, and a store there.
+__device__ __forceinline__ uint32_t map_rank(const void* p, uint32_t rank) {
+  uint32_t a;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_addr(p)), "r"(rank));
+  return a;
+}
+__device__ __forceinline__ void store_cluster(uint32_t addr, float v) {
+  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
+}
+
+template <int MODE>
+__global__ void __cluster_dims__(kCtas, 1, 1) __launch_bounds__(kThreads, 2)
+    linearize_split_kernel(const __grid_constant__ LinLaunch L) {
+  constexpr int NV = values(MODE);
+  __shared__ float val[kRound][NV][32];
+  __shared__ float red[kCtas][kAcc];  // the first CTA's receives every CTA's sums
+  __shared__ float mine[kAcc];
+  __shared__ ItemConst ic;
+  __shared__ int hits;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int it = blockIdx.x / kCtas;
+  const uint32_t w = cluster_rank();
+  const uint64_t pol = policy_evict_last_l();
+  int pair, begin, end;
+  tma::item_bounds(L, it, pair, begin, end);
+  if (threadIdx.x == 0) {
+    const PairDesc* pd = L.pairs ? L.pairs + pair : &L.single;
+    const MapDesc md = L.maps ? L.maps[pd->map] : L.single_map;
+    const SrcDesc sd = L.srcs ? L.srcs[pd->src] : L.single_src;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) ic.R[k] = pd->R[k];
+    ic.t[0] = pd->t[0];
+    ic.t[1] = pd->t[1];
+    ic.t[2] = pd->t[2];
+    ic.tmax = pd->tmax;
+    ic.inv_r = md.inv_r;
+    ic.margin_scale = md.margin_scale;
+    ic.mask = *md.vmask;
+    ic.vslots = md.vslots;
+    ic.pts = sd.pts;
+    ic.covs = sd.covs;
+    ic.pd = pd;
+    ic.r = md.r;
+    ic.max_probe = md.max_probe;
+    hits = 0;
+  }
+  if (threadIdx.x < kAcc) mine[threadIdx.x] = 0.0f;
+  __syncthreads();
+  Pose32 P;
+#pragma unroll
+  for (int k = 0; k < 9; ++k) P.R[k] = ic.R[k];
+  P.t[0] = ic.t[0];
+  P.t[1] = ic.t[1];
+  P.t[2] = ic.t[2];
+  P.tmax = ic.tmax;
+  MapDesc md;
+  md.vslots = ic.vslots;
+  md.inv_r = ic.inv_r;
+  md.margin_scale = ic.margin_scale;
+  md.r = ic.r;
+  md.max_probe = ic.max_probe;
+  const uint32_t mask = ic.mask;
+  const float* R = P.R;
+
+  float acc[kAcc];
+#pragma unroll
+  for (int k = 0; k < kAcc; ++k) acc[k] = 0.0f;
+  const int p0 = begin + (int)w * 32 + lane;
+  // points of the longest lane (lane 0)
+  const int n0 = end - begin - (int)w * 32;
+  const int steps = n0 > 0 ? (n0 + kSimpleThreads - 1) / kSimpleThreads : 0;
+  int my_hits = 0;
+  for (int j0 = 0; j0 < steps; j0 += kRound) {
+    // ---- kPer points per thread: key, first probe of each, resolve, terms ----
+    float x[kPer], y[kPer], z[kPer], c[kPer][6], q[kPer][3];
+    int kx[kPer], ky[kPer], kz[kPer];
+    uint32_t h[kPer], sa[kPer][8], sb[kPer][8];
+    unsigned long long key[kPer];
+    bool live[kPer];
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) {
+      const int64_t p = (int64_t)p0 + (int64_t)kSimpleThreads * (j0 + warp * kPer + u);
+      live[u] = p < end;
+      if (live[u]) {
+        const float* pt = ic.pts + 3 * p;
+        x[u] = __ldg(pt + 0);
+        y[u] = __ldg(pt + 1);
+        z[u] = __ldg(pt + 2);
+        const float2* cv = reinterpret_cast<const float2*>(ic.covs + 6 * p);
+        const float2 c01 = __ldg(cv + 0), c23 = __ldg(cv + 1), c45 = __ldg(cv + 2);
+        c[u][0] = c01.x; c[u][1] = c01.y; c[u][2] = c23.x;
+        c[u][3] = c23.y; c[u][4] = c45.x; c[u][5] = c45.y;
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) {
+      key[u] = kEmptyKey;
+      if (live[u]) {
+        q[u][0] = fmaf(R[0], x[u], fmaf(R[1], y[u], fmaf(R[2], z[u], P.t[0])));
+        q[u][1] = fmaf(R[3], x[u], fmaf(R[4], y[u], fmaf(R[5], z[u], P.t[1])));
+        q[u][2] = fmaf(R[6], x[u], fmaf(R[7], y[u], fmaf(R[8], z[u], P.t[2])));
+        source_key(P, ic.pd, md, x[u], y[u], z[u], q[u][0], q[u][1], q[u][2], kx[u], ky[u], kz[u]);
+        live[u] = key_in_range(kx[u]) && key_in_range(ky[u]) && key_in_range(kz[u]);
+      }
+      if (live[u]) {
+        key[u] = pack_key(kx[u], ky[u], kz[u]);
+        h[u] = hash_key(kx[u], ky[u], kz[u]) & mask;
+        ld_v8(md.vslots + h[u], pol, sa[u]);
+        ld_v8(reinterpret_cast<const char*>(md.vslots + h[u]) + 32, pol, sb[u]);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) {
+      bool hit = false;
+      if (live[u]) {
+        unsigned long long t = slot_key(sa[u]);
+        for (int p = 1; t != key[u] && t != kEmptyKey && (p > 1 || sa[u][kSlotSpill] != 0u) &&
+                        p < md.max_probe;
+             ++p) {
+          h[u] = (h[u] + 1) & mask;
+          ld_v8(md.vslots + h[u], pol, sa[u]);
+          ld_v8(reinterpret_cast<const char*>(md.vslots + h[u]) + 32, pol, sb[u]);
+          t = slot_key(sa[u]);
+        }
+        hit = t == key[u];
+      }
+      float v[NV];
+#pragma unroll
+      for (int k = 0; k < NV; ++k) v[k] = 0.0f;  // a miss adds zeros
+      if (hit) {
+        const float tx = __uint_as_float(sa[u][kSlotMu]) - q[u][0];
+        const float ty = __uint_as_float(sa[u][kSlotMu + 1]) - q[u][1];
+        const float tz = __uint_as_float(sa[u][kSlotMu + 2]) - q[u][2];
+        const float4 r1 = make_float4(__uint_as_float(sb[u][0]), __uint_as_float(sb[u][1]),
+                                      __uint_as_float(sb[u][2]), __uint_as_float(sb[u][3]));
+        const float4 r2 = make_float4(__uint_as_float(sb[u][4]), __uint_as_float(sb[u][5]), 0.f, 0.f);
+        const float d0 = fmaf(R[0], tx, fmaf(R[3], ty, R[6] * tz));
+        const float d1 = fmaf(R[1], tx, fmaf(R[4], ty, R[7] * tz));
+        const float d2 = fmaf(R[2], tx, fmaf(R[5], ty, R[8] * tz));
+        float m00, m01, m02, m11, m12, m22;
+        fused_cov(R, r1, r2, c[u], m00, m01, m02, m11, m12, m22);
+        const float i00 = fmaf(m11, m22, -m12 * m12);
+        const float i01 = fmaf(m02, m12, -m01 * m22);
+        const float i02 = fmaf(m01, m12, -m02 * m11);
+        const float i11 = fmaf(m00, m22, -m02 * m02);
+        const float i12 = fmaf(m01, m02, -m00 * m12);
+        const float i22 = fmaf(m00, m11, -m01 * m01);
+        const float det = fmaf(m00, i00, fmaf(m01, i01, m02 * i02));
+        const float sc = rcp_approx(det);
+        if (MODE == 0) {
+          const float w00 = __fmul_rn(i00, sc), w01 = __fmul_rn(i01, sc), w02 = __fmul_rn(i02, sc);
+          const float w11 = __fmul_rn(i11, sc), w12 = __fmul_rn(i12, sc), w22 = __fmul_rn(i22, sc);
+          v[0] = i00; v[1] = i01; v[2] = i02; v[3] = i11; v[4] = i12; v[5] = i22; v[6] = sc;
+          v[7] = fmaf(w00, d0, fmaf(w01, d1, w02 * d2));
+          v[8] = fmaf(w01, d0, fmaf(w11, d1, w12 * d2));
+          v[9] = fmaf(w02, d0, fmaf(w12, d1, w22 * d2));
+          v[10] = d0; v[11] = d1; v[12] = d2;
+          v[13] = x[u]; v[14] = y[u]; v[15] = z[u];
+        } else {
+          const float u0 = fmaf(i00, d0, fmaf(i01, d1, i02 * d2)) * sc;
+          const float u1 = fmaf(i01, d0, fmaf(i11, d1, i12 * d2)) * sc;
+          const float u2 = fmaf(i02, d0, fmaf(i12, d1, i22 * d2)) * sc;
+          v[0] = u0; v[1] = u1; v[2] = u2; v[3] = d0; v[4] = d1; v[5] = d2;
+          if (MODE >= 2) {
+            v[NV > 6 ? 6 : 0] = x[u]; v[NV > 6 ? 7 : 0] = y[u]; v[NV > 6 ? 8 : 0] = z[u];
+          }
+          if (MODE == 3) {
+            v[NV > 9 ? 9 : 0] = fmaf(c[u][0], u0, fmaf(c[u][1], u1, c[u][2] * u2));
+            v[NV > 9 ? 10 : 0] = fmaf(c[u][1], u0, fmaf(c[u][3], u1, c[u][4] * u2));
+            v[NV > 9 ? 11 : 0] = fmaf(c[u][2], u0, fmaf(c[u][4], u1, c[u][5] * u2));
+          }
+        }
+        ++my_hits;
+      }
+#pragma unroll
+      for (int k = 0; k < NV; ++k) val[warp * kPer + u][k][lane] = v[k];
+    }
+    __syncthreads();
+    // ---- the sums, point after point (the expressions of add_term / eval_term) ----
+    const int n = min(kRound, steps - j0);
+    if (MODE == 0) {
+      if (warp < 3) {
+        for (int j = 0; j < n; ++j) {
+          const float s = val[j][6][lane];
+          const float px = val[j][13][lane], py = val[j][14][lane], pz = val[j][15][lane];
+          const float w00 = __fmul_rn(val[j][0][lane], s), w01 = __fmul_rn(val[j][1][lane], s);
+          const float w02 = __fmul_rn(val[j][2][lane], s), w11 = __fmul_rn(val[j][3][lane], s);
+          const float w12 = __fmul_rn(val[j][4][lane], s), w22 = __fmul_rn(val[j][5][lane], s);
+          if (warp == 0) {
+            const float p00 = fmaf(py, w02, -pz * w01), p01 = fmaf(py, w12, -pz * w11),
+                        p02 = fmaf(py, w22, -pz * w12);
+            acc[6] += p00; acc[7] += p01; acc[8] += p02;
+            acc[0] = fmaf(p02, py, fmaf(-p01, pz, acc[0]));
+            acc[1] = fmaf(p00, pz, fmaf(-p02, px, acc[1]));
+            acc[2] = fmaf(p01, px, fmaf(-p00, py, acc[2]));
+          } else if (warp == 1) {
+            const float p10 = fmaf(pz, w00, -px * w02), p11 = fmaf(pz, w01, -px * w12),
+                        p12 = fmaf(pz, w02, -px * w22);
+            acc[9] += p10; acc[10] += p11; acc[11] += p12;
+            acc[3] = fmaf(p10, pz, fmaf(-p12, px, acc[3]));
+            acc[4] = fmaf(p11, px, fmaf(-p10, py, acc[4]));
+          } else {
+            const float p20 = fmaf(px, w01, -py * w00), p21 = fmaf(px, w11, -py * w01),
+                        p22 = fmaf(px, w12, -py * w02);
+            acc[12] += p20; acc[13] += p21; acc[14] += p22;
+            acc[5] = fmaf(p21, px, fmaf(-p20, py, acc[5]));
+          }
+        }
+      } else if (warp == 3) {
+        for (int j = 0; j < n; ++j) {
+          const float s = val[j][6][lane];
+#pragma unroll
+          for (int k = 0; k < 6; ++k)
+            acc[15 + k] = __fadd_rn(acc[15 + k], __fmul_rn(val[j][k][lane], s));
+        }
+      } else if (warp == 4) {
+        for (int j = 0; j < n; ++j) {
+          const float u0 = val[j][7][lane], u1 = val[j][8][lane], u2 = val[j][9][lane];
+          const float d0 = val[j][10][lane], d1 = val[j][11][lane], d2 = val[j][12][lane];
+          const float px = val[j][13][lane], py = val[j][14][lane], pz = val[j][15][lane];
+          acc[27] = fmaf(d0, u0, fmaf(d1, u1, fmaf(d2, u2, acc[27])));
+          acc[21] = fmaf(u1, pz, fmaf(-u2, py, acc[21]));
+          acc[22] = fmaf(u2, px, fmaf(-u0, pz, acc[22]));
+          acc[23] = fmaf(u0, py, fmaf(-u1, px, acc[23]));
+          acc[24] -= u0;
+          acc[25] -= u1;
+          acc[26] -= u2;
+        }
+      }
+    } else if (warp == 0) {
+      for (int j = 0; j < n; ++j) {
+        const float u0 = val[j][0][lane], u1 = val[j][1][lane], u2 = val[j][2][lane];
+        const float d0 = val[j][3][lane], d1 = val[j][4][lane], d2 = val[j][5][lane];
+        acc[6] = fmaf(d0, u0, fmaf(d1, u1, fmaf(d2, u2, acc[6])));
+        if (MODE >= 2) {
+          const float px = val[j][NV > 6 ? 6 : 0][lane], py = val[j][NV > 6 ? 7 : 0][lane],
+                      pz = val[j][NV > 6 ? 8 : 0][lane];
+          acc[0] = fmaf(2.0f * u1, pz, fmaf(-2.0f * u2, py, acc[0]));
+          acc[1] = fmaf(2.0f * u2, px, fmaf(-2.0f * u0, pz, acc[1]));
+          acc[2] = fmaf(2.0f * u0, py, fmaf(-2.0f * u1, px, acc[2]));
+          acc[3] -= 2.0f * u0;
+          acc[4] -= 2.0f * u1;
+          acc[5] -= 2.0f * u2;
+        }
+        if (MODE == 3) {
+          const float k0 = val[j][NV > 9 ? 9 : 0][lane], k1 = val[j][NV > 9 ? 10 : 0][lane],
+                      k2 = val[j][NV > 9 ? 11 : 0][lane];
+          acc[0] = fmaf(2.0f * u1, k2, fmaf(-2.0f * u2, k1, acc[0]));
+          acc[1] = fmaf(2.0f * u2, k0, fmaf(-2.0f * u0, k2, acc[1]));
+          acc[2] = fmaf(2.0f * u0, k1, fmaf(-2.0f * u1, k0, acc[2]));
+        }
+      }
+    }
+    __syncthreads();  // val is rewritten by the next round
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) my_hits += __shfl_xor_sync(0xFFFFFFFFu, my_hits, o);
+  if (lane == 0 && my_hits) atomicAdd(&hits, my_hits);
+  // the warp tree of the per-point kernel; an accumulator is nonzero in one warp only
+#pragma unroll
+  for (int k = 0; k < kAcc - 1; ++k) {
+    const int owner = MODE != 0 ? 0
+                      : k < 3 ? 0 : k < 5 ? 1 : k < 6 ? 2 : k < 9 ? 0 : k < 12 ? 1 : k < 15 ? 2
+                      : k < 21 ? 3 : 4;
+    if (MODE != 0 && k > 6) continue;
+    if (warp == owner) {
+      float v = acc[k];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
+      if (lane == 0) mine[k] = v;
+    }
+  }
+  cluster_sync();  // every CTA of the cluster runs, and its own sums are in place
+  if (threadIdx.x < kAcc)
+    store_cluster(map_rank(&red[w][threadIdx.x], 0),
+                  threadIdx.x == kAcc - 1 ? (float)hits : mine[threadIdx.x]);
+  cluster_sync();
+  if (w == 0 && threadIdx.x < kAcc) {
+    double s = 0.0;
+    for (int k = 0; k < kCtas; ++k) s += (double)red[k][threadIdx.x];
+    L.partials[(int64_t)it * kPartialStride + threadIdx.x] = s;
+  }
+}
+}  // namespace split
+
 // One warp per pair: lane k sums term k over the pair's items in order.  For the
 // gradient modes, an optional right Jacobian per pair (jr, 36 doubles, row-major)
 // maps the gradient g of the right perturbation to that of the pose increment,
@@ -1244,13 +1569,30 @@ int linearize_grid(int neighbours, int variant) {
   return device_sm_count() * VGICP_MIN_BLOCKS;
 }
 
+// Whether a launch goes to the cluster-per-item kernel: the per-point kernel's
+// results (variant 1), at least four points per thread in a full item, and at most
+// three items to four SMs.  Linearization with the per-pair sums, cluster per item
+// against per-point (items of 16K, factors of 20,000 points; 152 SMs): 2 items 27
+// against 71 us, 20 items 28 / 75, 40 items 38 / 75, 76 items 50 / 75, 120 items
+// 68 / 75, 152 items 79 / 75.
+static bool split_items(const LinLaunch& L, int variant) {
+  return L.neighbours != 27 && variant == 1 && L.mode <= 3 && L.grid <= 0 && !L.corr_out &&
+         !L.qkey_out && L.item_size >= 4 * kSimpleThreads && 4 * L.n_items <= 3 * device_sm_count();
+}
+
 int launch_linearize(const LinLaunch& L, cudaStream_t st) {
   if (L.n_items <= 0) return VGICP_OK;
   const int variant = L.mode != 0 ? 1 : (L.variant ? L.variant : default_variant());
   int grid = L.grid > 0 ? L.grid : linearize_grid(L.neighbours, variant);
   grid = std::min(grid, L.n_items);
   if (L.ev_start) VGICP_CUDA_TRY(cudaEventRecord(L.ev_start, st));
-  if (L.mode != 0) {
+  if (split_items(L, variant)) {
+    const unsigned ctas = (unsigned)L.n_items * split::kCtas;
+    if (L.mode == 0) split::linearize_split_kernel<0><<<ctas, split::kThreads, 0, st>>>(L);
+    else if (L.mode == 1) split::linearize_split_kernel<1><<<ctas, split::kThreads, 0, st>>>(L);
+    else if (L.mode == 2) split::linearize_split_kernel<2><<<ctas, split::kThreads, 0, st>>>(L);
+    else split::linearize_split_kernel<3><<<ctas, split::kThreads, 0, st>>>(L);
+  } else if (L.mode != 0) {
     // cost / gradient evaluations use the per-point kernel
     if (L.neighbours == 27) {
       if (L.mode == 1) launch_simple<27, 1>(L, grid, st);
