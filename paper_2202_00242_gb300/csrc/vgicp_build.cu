@@ -29,8 +29,8 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
-#include <mutex>
 #include <cstdint>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -416,126 +416,301 @@ __device__ __forceinline__ uint32_t spread10(uint32_t x) {
   x = (x | (x << 2)) & 0x09249249u;
   return x;
 }
-__device__ __forceinline__ uint32_t morton_of_key(unsigned long long key) {
-  const unsigned long long fm = (1ull << kKeyBits) - 1ull;
-  const uint32_t kx = (uint32_t)((key >> (2 * kKeyBits)) & fm);
-  const uint32_t ky = (uint32_t)((key >> kKeyBits) & fm);
-  const uint32_t kz = (uint32_t)(key & fm);
-  return spread10(kx) | (spread10(ky) << 1) | (spread10(kz) << 2);
-}
-
-// One CTA per (map, chunk): bitonic sort of the chunk's voxels by Morton code in
-// shared memory (ties by voxel id); vorder[rank] = v and gcount[rank] = the
-// voxel's point count.
+// One CTA (of 1024 threads) or one cluster of 8 CTAs (of 256) per (map, chunk): the
+// chunk's voxels sorted by Morton code (ties by voxel id); vorder[rank] = v and
+// gcount[rank] = the voxel's point count.
 //
-// Element i lives at i + i / 16 (one pad word per 16), which keeps every access
-// pattern below free of bank conflicts.  Each pass loads a group of up to 16
-// elements per thread into registers and applies up to four consecutive stages
-// of the network there: a group is the elements i0 + t s (t < 2^M), closed under
-// the strides s .. s 2^(M-1), so a merge level of stride 2^(p-1) .. 1 takes
-// ceil(p / 4) passes through shared memory instead of p.
-constexpr int kSortThreads = 1024;
-constexpr int kSortSmemElems = kMortonChunk + kMortonChunk / 16;
+// A stable radix sort, least significant digit first, the elements spread evenly
+// over the CTAs' shared memory.  A warp holds 32 J consecutive elements, J per lane
+// in registers; for each, the lanes with the same digit are found by one ballot per
+// digit bit, and the warp's counter of that digit gives the element's rank among the
+// warp's.  The CTAs exchange their digit counts through distributed shared memory; a
+// scan over (digit, CTA, warp) turns counters into places, and the elements are
+// scattered to the CTAs that own the places.  Up to 2,048 voxels are sorted by the
+// cluster's first CTA alone.
+// The code is shortened first: in each axis the bits above the largest magnitude
+// are copies of the sign (bit 9), which never decide an order by themselves, so
+// m + 1 bits per axis are sorted (a map within +-64 voxels: 21 bits, three passes of
+// 7) instead of 10.
+// Bounded by issue (about 60 instructions per element and pass) and, for few
+// chunks, by the passes' barriers; clusters pay for scattering between SMs, so many
+// chunks are sorted by one CTA each.  Cluster / single CTA, maps of n points (V
+// voxels): 10 maps of 20,000 (V = 19,000) 27 / 58 us, 10 of 20,000 (9,700) 17 / 36,
+// 20 of 40,000 (37,000) 56 / 58, 20 of 80,000 (41,000) 52 / 49, 100 of 50,000
+// (12,000) 76 / 47, 500 of 50,000 264 / 169.  A bitonic sort (29 passes through shared
+// memory for 16K elements) took 65 us for 10 maps of 20,000 and 278 us for the 500
+// maps of the global map.
+constexpr int kDigitBits = 8;
+constexpr int kDigits = 1 << kDigitBits;
+constexpr int kSortElems = 2048;  // elements a CTA of a cluster holds
 
-__device__ __forceinline__ uint32_t sort_phys(uint32_t i) { return i + (i >> 4); }
+template <int CTAS, int THREADS>
+struct SortSmem {
+  static constexpr int kWarps = THREADS / 32, kGroups = THREADS / kDigits;
+  uint32_t key[kMortonChunk / CTAS];
+  uint16_t idx[kMortonChunk / CTAS];
+  uint32_t count[kWarps][kDigits];   // then: place of the warp's first of the digit
+  uint32_t part[kGroups][kDigits];   // the same per 8 warps
+  uint32_t total[CTAS][kDigits];     // digit counts of every CTA of the cluster
+  uint32_t bits[CTAS];
+  uint32_t warp[kWarps];
+};
 
-__device__ __forceinline__ void cmp_swap(unsigned long long& a, unsigned long long& b, bool up) {
-  if ((a > b) == up) {
-    const unsigned long long t = a;
-    a = b;
-    b = t;
-  }
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::
+                   : "memory");
+}
+__device__ __forceinline__ uint32_t smem_of_rank(const void* p, uint32_t rank) {
+  uint32_t a;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;"
+               : "=r"(a)
+               : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+  return a;
+}
+__device__ __forceinline__ void st_cluster(uint32_t addr, uint32_t v) {
+  asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+__device__ __forceinline__ void st_cluster16(uint32_t addr, uint32_t v) {
+  asm volatile("st.shared::cluster.u16 [%0], %1;" ::"r"(addr), "h"((uint16_t)v) : "memory");
 }
 
-// The stages of strides s 2^(M-1) .. s of merge level k on every group.
-template <int M>
-__device__ __forceinline__ void bitonic_pass(unsigned long long* sk, uint32_t N, uint32_t k,
-                                             uint32_t s_log) {
-  constexpr int G = 1 << M;
-  const uint32_t s = 1u << s_log;
-  for (uint32_t g = threadIdx.x; g < (N >> M); g += blockDim.x) {
-    const uint32_t i0 = ((g >> s_log) << (s_log + M)) | (g & (s - 1u));
-    const bool up = (i0 & k) == 0u;  // the same for the whole group (its bits are below k)
-    unsigned long long r[G];
-#pragma unroll
-    for (int t = 0; t < G; ++t) r[t] = sk[sort_phys(i0 + (uint32_t)t * s)];
-#pragma unroll
-    for (int j = G >> 1; j > 0; j >>= 1)
-#pragma unroll
-      for (int t = 0; t < G; ++t)
-        if ((t ^ j) > t) cmp_swap(r[t], r[t ^ j], up);
-#pragma unroll
-    for (int t = 0; t < G; ++t) sk[sort_phys(i0 + (uint32_t)t * s)] = r[t];
-  }
-}
-
-__global__ void __launch_bounds__(kSortThreads) morton_sort_kernel(
+template <int CTAS, int THREADS>
+__global__ void __launch_bounds__(THREADS) morton_sort_kernel(
     const int2* __restrict__ chunks, const uint32_t* __restrict__ vbase,
     const unsigned long long* __restrict__ vkeys, const uint32_t* __restrict__ vcount,
     uint32_t* __restrict__ vorder, uint32_t* __restrict__ gcount) {
-  extern __shared__ unsigned long long sk[];
-  const int m = chunks[blockIdx.x].x;
-  const uint32_t V = vbase[m + 1] - vbase[m];
-  const uint32_t lo = (uint32_t)chunks[blockIdx.x].y * kMortonChunk;
+  constexpr int kWarps = THREADS / 32, kGroups = THREADS / kDigits, kEach = kWarps / kGroups;
+  constexpr int kItems = kMortonChunk / (CTAS * THREADS);
+  static_assert(kEach == 8 && kItems % 2 == 0, "scan and register layout");
+  extern __shared__ __align__(16) unsigned char sort_smem[];
+  auto& S = *reinterpret_cast<SortSmem<CTAS, THREADS>*>(sort_smem);
+  const int2 ch = chunks[blockIdx.x / CTAS];
+  const int m = ch.x;
+  const uint32_t v0 = vbase[m], V = vbase[m + 1] - v0;
+  const uint32_t lo = (uint32_t)ch.y * kMortonChunk;
   if (lo >= V) return;
   const uint32_t cnt = min((uint32_t)kMortonChunk, V - lo);
-#ifdef VGICP_NO_MORTON
-  for (uint32_t i = threadIdx.x; i < cnt; i += blockDim.x) {
-    vorder[vbase[m] + lo + i] = vbase[m] + lo + i;
-    gcount[vbase[m] + lo + i] = vcount[vbase[m] + lo + i];
-  }
-  return;
-#endif
-  uint32_t N = 16;  // at least one full register group
-  while (N < cnt) N <<= 1;
-  const uint32_t first = vbase[m] + lo;
-  for (uint32_t i = threadIdx.x; i < N; i += blockDim.x)
-    sk[sort_phys(i)] =
-        i < cnt ? (((unsigned long long)morton_of_key(vkeys[first + i]) << 32) | i) : ~0ull;
-  __syncthreads();
-  // levels k = 2 .. 16: inside blocks of 16 consecutive elements
-  for (uint32_t g = threadIdx.x; g < (N >> 4); g += blockDim.x) {
-    unsigned long long r[16];
+  const uint32_t first = v0 + lo;
+  const uint32_t rank = CTAS > 1 ? cluster_rank() : 0u;
+  const uint32_t ctas = cnt <= (uint32_t)kSortElems ? 1u : (uint32_t)CTAS;
+  if (rank >= ctas) return;  // the first CTA sorts alone: no cluster barrier below
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const uint32_t J = (cnt + ctas * THREADS - 1) / (ctas * THREADS);  // elements per lane
+  const uint32_t c0 = rank * (J * THREADS);                          // this CTA's first
+  const uint32_t mine = cnt > c0 ? min(J * (uint32_t)THREADS, cnt - c0) : 0u;
+  const uint32_t e0 = (uint32_t)w * 32u * J + (uint32_t)lane;  // element j: c0 + e0 + 32 j
+
+  // keys: 10 bits per axis, and the bits that differ from their axis' sign
+  uint32_t key[kItems];
+  uint32_t diff = 0u;
 #pragma unroll
-    for (int t = 0; t < 16; ++t) r[t] = sk[sort_phys(16u * g + t)];
-#pragma unroll
-    for (int k = 2; k <= 16; k <<= 1)
-#pragma unroll
-      for (int j = k >> 1; j > 0; j >>= 1)
-#pragma unroll
-        for (int t = 0; t < 16; ++t)
-          if ((t ^ j) > t) cmp_swap(r[t], r[t ^ j], ((16u * g + t) & (uint32_t)k) == 0u);
-#pragma unroll
-    for (int t = 0; t < 16; ++t) sk[sort_phys(16u * g + t)] = r[t];
-  }
-  __syncthreads();
-  // levels k = 32 .. N: strides 2^(p-1) .. 1 in passes of up to four, the
-  // partial pass (p mod 4 strides) first
-  for (uint32_t p = 5; (1u << p) <= N; ++p) {
-    const uint32_t k = 1u << p;
-    int top = (int)p - 1;  // log2 of the largest stride not yet applied
-    const int rem = (int)(p & 3u);
-    if (rem) {
-      const uint32_t s_log = (uint32_t)(top - rem + 1);
-      if (rem == 1) bitonic_pass<1>(sk, N, k, s_log);
-      else if (rem == 2) bitonic_pass<2>(sk, N, k, s_log);
-      else bitonic_pass<3>(sk, N, k, s_log);
-      top -= rem;
-      __syncthreads();
-    }
-    for (; top >= 0; top -= 4) {
-      bitonic_pass<4>(sk, N, k, (uint32_t)(top - 3));
-      __syncthreads();
+  for (int j = 0; j < kItems; ++j) {
+    const uint32_t e = e0 + 32u * j;
+    key[j] = 0u;
+    if (j < (int)J && e < mine) {
+      const unsigned long long k = vkeys[first + c0 + e];
+      const uint32_t x = (uint32_t)(k >> (2 * kKeyBits)) & 1023u, y = (uint32_t)(k >> kKeyBits) & 1023u,
+                     z = (uint32_t)k & 1023u;
+      key[j] = x | (y << 10) | (z << 20);
+      diff |= (x ^ (0u - (x >> 9))) | (y ^ (0u - (y >> 9))) | (z ^ (0u - (z >> 9)));
     }
   }
-  for (uint32_t i = threadIdx.x; i < cnt; i += blockDim.x) {
-    const uint32_t v = first + (uint32_t)(sk[sort_phys(i)] & 0xFFFFFFFFull);
-    vorder[first + i] = v;
-    gcount[first + i] = vcount[v];
+  diff = __reduce_or_sync(0xFFFFFFFFu, diff & 511u);
+  if (lane == 0) S.warp[w] = diff;
+  __syncthreads();
+  uint32_t bits = 0u;
+  for (int i = 0; i < kWarps; ++i) bits |= S.warp[i];
+  if (ctas > 1u) {
+    cluster_sync();  // every CTA of the cluster runs
+    if (threadIdx.x < ctas) st_cluster(smem_of_rank(&S.bits[rank], threadIdx.x), bits);
+    cluster_sync();
+    for (uint32_t i = 0; i < ctas; ++i) bits |= S.bits[i];
+  }
+  const int mag = 32 - __clz((int)bits);               // magnitude bits kept (0 .. 9)
+  const int total_bits = 3 * (mag + 1);
+  const int passes = (total_bits + kDigitBits - 1) / kDigitBits;
+  const int digit_bits = (total_bits + passes - 1) / passes;
+  const uint32_t low = (1u << mag) - 1u;
+#pragma unroll
+  for (int j = 0; j < kItems; ++j) {
+    const uint32_t x = key[j] & 1023u, y = (key[j] >> 10) & 1023u, z = key[j] >> 20;
+    key[j] = spread10((x & low) | ((x >> 9) << mag)) | (spread10((y & low) | ((y >> 9) << mag)) << 1) |
+             (spread10((z & low) | ((z >> 9) << mag)) << 2);
+  }
+  uint32_t idx[kItems / 2];  // index in the chunk, two 16-bit values a word
+#pragma unroll
+  for (int j = 0; j < kItems; j += 2) {
+    const uint32_t i = c0 + e0 + 32u * j;
+    idx[j / 2] = i | ((i + 32u) << 16);
+  }
+
+  const uint32_t digit_mask = (1u << digit_bits) - 1u;
+  const uint32_t lower = (1u << lane) - 1u;
+  const uint32_t inv_j = 65536u / J + 1u;  // (p / 256) / J for p / 256 < 64 and J <= 8
+  for (int pass = 0; pass < passes; ++pass) {
+    const int shift = pass * digit_bits;
+    if (pass > 0) {
+#pragma unroll
+      for (int j = 0; j < kItems; ++j) {
+        const uint32_t e = e0 + 32u * j;
+        if (j < (int)J && e < mine) {
+          key[j] = S.key[e];
+          const uint32_t v = S.idx[e];
+          idx[j / 2] = (j & 1) ? (idx[j / 2] & 0xFFFFu) | (v << 16) : (idx[j / 2] & 0xFFFF0000u) | v;
+        }
+      }
+    }
+    for (int d = lane; d < kDigits; d += 32) S.count[w][d] = 0u;
+    __syncwarp();
+    uint32_t rk[kItems / 2];  // rank among the warp's elements of the digit, 16 bits
+#pragma unroll
+    for (int j = 0; j < kItems; ++j) {
+      if (j < (int)J) {  // the same for all lanes
+        const bool live = e0 + 32u * j < mine;
+        const uint32_t d = (key[j] >> shift) & digit_mask;
+        uint32_t peers = __ballot_sync(0xFFFFFFFFu, live);
+#pragma unroll
+        for (int b = 0; b < kDigitBits; ++b) {
+          const uint32_t bit = 0u - ((d >> b) & 1u);
+          peers &= ~(__ballot_sync(0xFFFFFFFFu, bit != 0u) ^ bit);
+        }
+        const uint32_t seen = live ? S.count[w][d] : 0u;
+        __syncwarp();
+        if (live && (peers & lower) == 0u) S.count[w][d] = seen + (uint32_t)__popc(peers);
+        __syncwarp();
+        const uint32_t r = seen + (uint32_t)__popc(peers & lower);
+        rk[j / 2] = (j & 1) ? rk[j / 2] | (r << 16) : r;
+      }
+    }
+    __syncthreads();
+    // counters -> places, in the order (digit, CTA, warp); thread = (digit, 8 warps)
+    const int d = threadIdx.x % kDigits, g = threadIdx.x / kDigits;
+    uint32_t c[kEach], sum = 0u;
+#pragma unroll
+    for (int i = 0; i < kEach; ++i) {
+      c[i] = S.count[g * kEach + i][d];
+      sum += c[i];
+    }
+    if (kGroups > 1) {
+      S.part[g][d] = sum;
+      __syncthreads();
+      if (g == 0)
+#pragma unroll
+        for (int i = 1; i < kGroups; ++i) sum += S.part[i][d];
+    }
+    uint32_t all = sum, before = 0u, inc = 0u;  // of the digit (threads of group 0)
+    if (ctas > 1u) {
+      for (uint32_t r = 0; r < ctas; ++r) st_cluster(smem_of_rank(&S.total[rank][d], r), sum);
+      cluster_sync();
+      all = 0u;
+#pragma unroll
+      for (int r = 0; r < CTAS; ++r) {
+        const uint32_t t = S.total[r][d];
+        all += t;
+        if (r < (int)rank) before += t;
+      }
+    }
+    if (g == 0) {  // whole warps
+      inc = all;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, inc, o);
+        if (lane >= o) inc += y;
+      }
+      if (lane == 31) S.warp[w] = inc;
+    }
+    __syncthreads();
+    uint32_t run = 0u;
+    if (g == 0) {
+      run = inc - all + before;
+      for (int i = 0; i < w; ++i) run += S.warp[i];
+    }
+    if (kGroups > 1) {
+      if (g == 0) {  // part <- first place of (digit, group)
+        const uint32_t p0 = c[0] + c[1] + c[2] + c[3] + c[4] + c[5] + c[6] + c[7];
+        uint32_t at = run + p0;
+#pragma unroll
+        for (int i = 1; i < kGroups; ++i) {
+          const uint32_t x = S.part[i][d];
+          S.part[i][d] = at;
+          at += x;
+        }
+      }
+      __syncthreads();
+      if (g > 0) run = S.part[g][d];
+    }
+#pragma unroll
+    for (int i = 0; i < kEach; ++i) {
+      S.count[g * kEach + i][d] = run;
+      run += c[i];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < kItems; ++j) {
+      if (j < (int)J && e0 + 32u * j < mine) {
+        const uint32_t p = S.count[w][(key[j] >> shift) & digit_mask] +
+                           ((rk[j / 2] >> (16 * (j & 1))) & 0xFFFFu);
+        const uint32_t i = (idx[j / 2] >> (16 * (j & 1))) & 0xFFFFu;
+        if (CTAS == 1 || ctas == 1u) {
+          S.key[p] = key[j];
+          S.idx[p] = (uint16_t)i;
+        } else {
+          const uint32_t to = ((p / THREADS) * inv_j) >> 16;
+          const uint32_t o = p - to * (J * THREADS);
+          st_cluster(smem_of_rank(&S.key[o], to), key[j]);
+          st_cluster16(smem_of_rank(&S.idx[o], to), i);
+        }
+      }
+    }
+    if (ctas > 1u) cluster_sync();
+    else __syncthreads();
+  }
+  for (uint32_t i = threadIdx.x; i < mine; i += THREADS) {
+    const uint32_t v = first + (uint32_t)S.idx[i];
+    vorder[first + c0 + i] = v;
+    gcount[first + c0 + i] = vcount[v];
   }
 }
 
-
+// Launches the sort with CTAS CTAs of THREADS threads per chunk.
+template <int CTAS, int THREADS>
+int launch_sort(const MapSet* s, uint32_t* vorder, uint32_t* gcount, cudaStream_t st) {
+  constexpr int kBytes = (int)sizeof(SortSmem<CTAS, THREADS>);
+  auto* kernel = morton_sort_kernel<CTAS, THREADS>;
+  if (kBytes > 48 * 1024) {  // above the default limit: opt in once per device
+    static std::mutex attr_mu;
+    static bool attr_set[kMaxDevices] = {false};
+    int dev = 0;
+    VGICP_CUDA_TRY(cudaGetDevice(&dev));
+    if (dev < 0 || dev >= kMaxDevices)
+      return set_error(VGICP_ERR_INVALID_ARG, "device index beyond the supported range");
+    std::lock_guard<std::mutex> lock(attr_mu);
+    if (!attr_set[dev]) {
+      VGICP_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kBytes));
+      attr_set[dev] = true;
+    }
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)s->n_chunks * CTAS);
+  cfg.blockDim = dim3(THREADS);
+  cfg.dynamicSmemBytes = kBytes;
+  cfg.stream = st;
+  cudaLaunchAttribute attr = {};
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = CTAS;
+  attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = CTAS > 1 ? 1 : 0;
+  VGICP_CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel, (const int2*)s->d_chunks, (const uint32_t*)s->d_vbase,
+                                    (const unsigned long long*)s->d_vkeys,
+                                    (const uint32_t*)s->d_vcount, vorder, gcount));
+  return VGICP_OK;
+}
 
 __device__ __forceinline__ uint32_t lookup_capacity(uint32_t nvox) {
   uint32_t c = 16;
@@ -894,24 +1069,11 @@ int launch_build(MapSet* s, const float* points, const float* covs, cudaStream_t
   // the lists' (base << 32 | fill) words, by voxel: in the record storage, which
   // finalize fills only after the scatter (8 of its 48 B per voxel)
   unsigned long long* bfill = reinterpret_cast<unsigned long long*>(s->d_recs);
-  {
-    // the sort's shared memory is above the default limit: opt in once per device
-    static std::mutex attr_mu;
-    static bool attr_set[kMaxDevices] = {false};
-    int dev = 0;
-    VGICP_CUDA_TRY(cudaGetDevice(&dev));
-    if (dev < 0 || dev >= kMaxDevices)
-      return set_error(VGICP_ERR_INVALID_ARG, "device index beyond the supported range");
-    std::lock_guard<std::mutex> lock(attr_mu);
-    if (!attr_set[dev]) {
-      VGICP_CUDA_TRY(cudaFuncSetAttribute(morton_sort_kernel,
-                                          cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)(sizeof(unsigned long long) * kSortSmemElems)));
-      attr_set[dev] = true;
-    }
-  }
-  morton_sort_kernel<<<s->n_chunks, kSortThreads, sizeof(unsigned long long) * kSortSmemElems,
-                       st>>>(s->d_chunks, s->d_vbase, s->d_vkeys, s->d_vcount, vorder, gcount);
+  // a cluster per chunk while that leaves two SMs or more to a chunk (figures at the
+  // kernel)
+  rc = 2 * s->n_chunks <= device_sm_count() ? launch_sort<8, 256>(s, vorder, gcount, st)
+                                            : launch_sort<1, 1024>(s, vorder, gcount, st);
+  if (rc != VGICP_OK) return rc;
   VGICP_CUDA_TRY(cudaGetLastError());
   // list offsets in rank order, and by voxel
   {
