@@ -268,6 +268,86 @@ __device__ __forceinline__ int map_of_rank(const uint32_t* __restrict__ vbase, i
   return lo;
 }
 
+// Exact sums of list entries o + first, o + first + step, ... < o + c of the grouped
+// cloud (plain loads: written by the caller's kernel), in double-float: hi + lo stays
+// the exact sum while each TwoSum error adds exactly to lo (checked).
+__device__ __forceinline__ void sum_entries(const float* gpts, const float* gcovs, uint32_t o,
+                                            uint32_t c, uint32_t first, uint32_t step, float* hi,
+                                            float* lo, bool& exact) {
+  for (uint32_t a = first; a < c; a += step) {
+    const int64_t d = (int64_t)o + a;
+    float f[9];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) f[k] = gpts[3 * d + k];
+    const float2* gc = reinterpret_cast<const float2*>(gcovs + 6 * d);
+    const float2 c0 = gc[0], c1 = gc[1], c2 = gc[2];
+    f[3] = c0.x; f[4] = c0.y; f[5] = c1.x; f[6] = c1.y; f[7] = c2.x; f[8] = c2.y;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+      float t, e, u, e2;
+      two_sum(hi[k], f[k], t, e);
+      two_sum(lo[k], e, u, e2);
+      exact = exact && (e2 == 0.0f);
+      hi[k] = t;
+      lo[k] = u;
+    }
+  }
+}
+
+// The record of voxel v (c points at o of the grouped cloud) from its sums; q: the
+// means of the nine components.
+__device__ __forceinline__ void write_record(uint32_t v, uint32_t o, uint32_t c, float* hi,
+                                             float* lo, bool exact, const float* gpts,
+                                             const float* gcovs, float4* __restrict__ recs,
+                                             float* q) {
+#pragma unroll
+  for (int k = 0; k < 9; ++k) {  // hi = RN(hi + lo), lo = the exact remainder
+    float t, e;
+    two_sum(hi[k], lo[k], t, e);
+    hi[k] = t;
+    lo[k] = e;
+  }
+  // q = RN32(RN64(sum / N)) per component: from the exact float pair in
+  // float32 where certified, else (rare) from the binary64 definition
+  uint32_t need64 = exact ? 0u : 0x1FFu;
+  if (exact) {
+    const float rN = __frcp_rn((float)c);
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+      bool ok;
+      q[k] = mean_rn32(hi[k], lo[k], c, rN, ok);
+      if (!ok) need64 |= 1u << k;
+    }
+  }
+  if (need64) {
+    double sum[9];
+    if (exact) {
+#pragma unroll
+      for (int k = 0; k < 9; ++k) sum[k] = __dadd_rn((double)hi[k], (double)lo[k]);  // exact
+    } else {
+      // binary64 sum in ascending point index (the grouped order; rare: large
+      // dynamic range)
+#pragma unroll
+      for (int k = 0; k < 9; ++k) sum[k] = 0.0;
+      for (uint32_t a = 0; a < c; ++a) {
+        const int64_t d = (int64_t)o + a;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) sum[k] = __dadd_rn(sum[k], (double)gpts[3 * d + k]);
+#pragma unroll
+        for (int k = 0; k < 6; ++k) sum[3 + k] = __dadd_rn(sum[3 + k], (double)gcovs[6 * d + k]);
+      }
+    }
+    const double N = (double)c;
+    const double y = __drcp_rn(N);
+#pragma unroll
+    for (int k = 0; k < 9; ++k)
+      if (need64 & (1u << k)) q[k] = __double2float_rn(div_rn(sum[k], N, y));
+  }
+  recs[3 * v + 0] = make_float4(q[0], q[1], q[2], __uint_as_float(c));
+  recs[3 * v + 1] = make_float4(q[3], q[4], q[5], q[6]);
+  recs[3 * v + 2] = make_float4(q[7], q[8], 0.0f, 0.0f);
+}
+
 __global__ void __launch_bounds__(kFinThreads) finalize_kernel(
     int64_t n_max, const uint32_t* __restrict__ n_vox, const uint32_t* __restrict__ n_valid,
     const float* __restrict__ pts, const float* __restrict__ covs,
@@ -325,77 +405,12 @@ __global__ void __launch_bounds__(kFinThreads) finalize_kernel(
     __syncthreads();  // the CTA's global writes are visible to the CTA after this
     // 3. sums from the grouped copy (plain loads: written by this kernel)
     if (mine) {
-      float hi[9], lo[9];
+      float hi[9], lo[9], q[9];
 #pragma unroll
       for (int k = 0; k < 9; ++k) hi[k] = lo[k] = 0.0f;
       bool exact = true;
-      for (uint32_t a = 0; a < c; ++a) {
-        const int64_t d = (int64_t)o + a;
-        float f[9];
-#pragma unroll
-        for (int k = 0; k < 3; ++k) f[k] = gpts[3 * d + k];
-        const float2* gc = reinterpret_cast<const float2*>(gcovs + 6 * d);
-        const float2 c0 = gc[0], c1 = gc[1], c2 = gc[2];
-        f[3] = c0.x; f[4] = c0.y; f[5] = c1.x; f[6] = c1.y; f[7] = c2.x; f[8] = c2.y;
-        // hi + lo stays the exact sum while each TwoSum error adds exactly to lo
-        // (checked); renormalised once at the end
-#pragma unroll
-        for (int k = 0; k < 9; ++k) {
-          float t, e, u, e2;
-          two_sum(hi[k], f[k], t, e);
-          two_sum(lo[k], e, u, e2);
-          exact = exact && (e2 == 0.0f);
-          hi[k] = t;
-          lo[k] = u;
-        }
-      }
-#pragma unroll
-      for (int k = 0; k < 9; ++k) {  // hi = RN(hi + lo), lo = the exact remainder
-        float t, e;
-        two_sum(hi[k], lo[k], t, e);
-        hi[k] = t;
-        lo[k] = e;
-      }
-      // q = RN32(RN64(sum / N)) per component: from the exact float pair in
-      // float32 where certified, else (rare) from the binary64 definition
-      float q[9];
-      uint32_t need64 = exact ? 0u : 0x1FFu;
-      if (exact) {
-        const float rN = __frcp_rn((float)c);
-#pragma unroll
-        for (int k = 0; k < 9; ++k) {
-          bool ok;
-          q[k] = mean_rn32(hi[k], lo[k], c, rN, ok);
-          if (!ok) need64 |= 1u << k;
-        }
-      }
-      if (need64) {
-        double sum[9];
-        if (exact) {
-#pragma unroll
-          for (int k = 0; k < 9; ++k) sum[k] = __dadd_rn((double)hi[k], (double)lo[k]);  // exact
-        } else {
-          // binary64 sum in ascending point index (the grouped order; rare: large
-          // dynamic range)
-#pragma unroll
-          for (int k = 0; k < 9; ++k) sum[k] = 0.0;
-          for (uint32_t a = 0; a < c; ++a) {
-            const int64_t d = (int64_t)o + a;
-#pragma unroll
-            for (int k = 0; k < 3; ++k) sum[k] = __dadd_rn(sum[k], (double)gpts[3 * d + k]);
-#pragma unroll
-            for (int k = 0; k < 6; ++k) sum[3 + k] = __dadd_rn(sum[3 + k], (double)gcovs[6 * d + k]);
-          }
-        }
-        const double N = (double)c;
-        const double y = __drcp_rn(N);
-#pragma unroll
-        for (int k = 0; k < 9; ++k)
-          if (need64 & (1u << k)) q[k] = __double2float_rn(div_rn(sum[k], N, y));
-      }
-      recs[3 * v + 0] = make_float4(q[0], q[1], q[2], __uint_as_float(c));
-      recs[3 * v + 1] = make_float4(q[3], q[4], q[5], q[6]);
-      recs[3 * v + 2] = make_float4(q[7], q[8], 0.0f, 0.0f);
+      sum_entries(gpts, gcovs, o, c, 0u, 1u, hi, lo, exact);
+      write_record(v, o, c, hi, lo, exact, gpts, gcovs, recs, q);
       // the voxel's map (ranks and voxel ids of a map share its range
       // [vbase[m], vbase[m + 1])): a CTA's ranks rarely span two maps
       int m = seg_map[0];
@@ -404,6 +419,137 @@ __global__ void __launch_bounds__(kFinThreads) finalize_kernel(
                     lslot_of, status);
     }
     __syncthreads();  // the stage is reused by the next batch
+  }
+}
+
+// (hi, lo) += the same of the lane at distance `delta`, exactly (checked).
+__device__ __forceinline__ void add_lane(float* hi, float* lo, bool& exact, int delta) {
+  const bool other = __shfl_xor_sync(0xFFFFFFFFu, (int)exact, delta) != 0;
+  exact = exact && other;
+#pragma unroll
+  for (int k = 0; k < 9; ++k) {
+    const float h = __shfl_xor_sync(0xFFFFFFFFu, hi[k], delta);
+    const float l = __shfl_xor_sync(0xFFFFFFFFu, lo[k], delta);
+    float t, e, u, e2, v, e3;
+    two_sum(hi[k], h, t, e);
+    two_sum(lo[k], l, u, e2);
+    two_sum(u, e, v, e3);
+    exact = exact && e2 == 0.0f && e3 == 0.0f;
+    hi[k] = t;
+    lo[k] = v;
+  }
+}
+
+// The same for long lists: R consecutive ranks per CTA, 128 / R threads per voxel, R
+// the power of two that makes about 512 points per CTA.  The lists are not sorted
+// first: a point's position in the grouped cloud is the number of smaller indices in
+// its list, counted by the thread that copies it.  A voxel's threads sum its points
+// (exact partial sums, joined exactly); a list longer than 64 points per thread is
+// summed by the whole warp.  A segment longer than the staging buffer (a voxel of
+// thousands of points) is sorted in place by one thread per voxel, as above.
+// Bounded by the latency of the chain offsets - indices - gather - sums on few CTAs.
+// This kernel / the one above (points per voxel on average): ten maps of 20,000
+// points 19 / 18 us (2.0), 20 / 28 (5.7), 19 / 55 (11), 21 / 148 (23), 49 / 1554 (91);
+// 20 maps of 40,000 52 / 66 (11); 100 maps of 50,000 252 / 230 (3.8), 226 / 212 (8.1),
+// 233 / 314 (15), 322 / 781 (33).  More registers (80 against 56) cost it the large
+// sets of short lists.
+constexpr uint32_t kFinSerial = 64;
+__global__ void __launch_bounds__(kFinThreads) finalize_long_kernel(
+    int64_t n_max, const uint32_t* __restrict__ n_vox, const uint32_t* __restrict__ n_valid,
+    const float* __restrict__ pts, const float* __restrict__ covs,
+    const uint32_t* __restrict__ vorder, const uint32_t* __restrict__ goff,
+    uint32_t* __restrict__ plist, float4* __restrict__ recs, float* gpts, float* gcovs,
+    const unsigned long long* __restrict__ vkeys, int32_t n_maps,
+    const uint32_t* __restrict__ vbase, const int64_t* __restrict__ slot_base,
+    const uint32_t* __restrict__ vmask, int32_t max_probe, VSlot* vslots,
+    uint32_t* __restrict__ lslot_of, int32_t* status) {
+  __shared__ uint32_t stage[kFinStage];
+  __shared__ uint32_t list_at[kFinThreads];  // first entry of each list, in the segment
+  const int64_t V = min((int64_t)*n_vox, n_max);
+  const uint32_t total = *n_valid;  // end of the last list (goff[V] is not stored)
+  const uint32_t avg = (uint32_t)((int64_t)total / max((int64_t)1, V));
+  int R = kFinThreads;
+  while (R > 4 && (uint32_t)R * avg > 512u) R >>= 1;
+  const int per = kFinThreads / R;  // threads per voxel (1 .. 32)
+  const int lane = threadIdx.x & 31, part = (int)threadIdx.x & (per - 1);
+  for (int64_t r0 = (int64_t)blockIdx.x * R; r0 < V; r0 += (int64_t)gridDim.x * R) {
+    const int64_t r1 = min(V, r0 + R);
+    const uint32_t seg0 = goff[r0];
+    const uint32_t seg1 = r1 < V ? goff[r1] : total;
+    const uint32_t len = seg1 - seg0;
+    const bool staged = len <= (uint32_t)kFinStage;
+    const int64_t r = r0 + (int)threadIdx.x / per;
+    const bool ours = r < r1, mine = ours && part == 0;
+    const uint32_t v = mine ? vorder[r] : 0u;
+    const uint32_t o = ours ? goff[r] : 0u;
+    const uint32_t c = ours ? (r + 1 < V ? goff[r + 1] : total) - o : 0u;
+    if (staged) {
+      for (uint32_t i = threadIdx.x; i < len; i += kFinThreads) stage[i] = plist[seg0 + i];
+      if (mine) list_at[r - r0] = o - seg0;
+    } else if (mine) {
+      insertion_sort(plist + o, c);
+    }
+    __syncthreads();
+    for (uint32_t i = threadIdx.x; i < len; i += kFinThreads) {
+      const uint32_t id = staged ? stage[i] : plist[seg0 + i];
+      const int64_t j = id;
+      const float x = __ldg(pts + 3 * j), y = __ldg(pts + 3 * j + 1), z = __ldg(pts + 3 * j + 2);
+      const float2* cv = reinterpret_cast<const float2*>(covs + 6 * j);
+      const float2 c0 = __ldg(cv), c1 = __ldg(cv + 1), c2 = __ldg(cv + 2);
+      int64_t d = (int64_t)seg0 + i;
+      if (staged) {
+        int q = 0, end = (int)(r1 - r0);  // the entry's list: the last with list_at <= i
+        while (end - q > 1) {
+          const int mid = (q + end) >> 1;
+          if (list_at[mid] <= i) q = mid; else end = mid;
+        }
+        const uint32_t a = list_at[q], e = q + 1 < (int)(r1 - r0) ? list_at[q + 1] : len;
+        uint32_t smaller = 0u;
+#pragma unroll 4
+        for (uint32_t t = a; t < e; ++t) smaller += stage[t] < id ? 1u : 0u;
+        d = (int64_t)seg0 + a + smaller;
+      }
+      gpts[3 * d + 0] = x;
+      gpts[3 * d + 1] = y;
+      gpts[3 * d + 2] = z;
+      float2* gc = reinterpret_cast<float2*>(gcovs + 6 * d);
+      gc[0] = c0;
+      gc[1] = c1;
+      gc[2] = c2;
+    }
+    __syncthreads();  // the CTA's global writes are visible to the CTA after this
+    float hi[9], lo[9], q[9];
+#pragma unroll
+    for (int k = 0; k < 9; ++k) hi[k] = lo[k] = 0.0f;
+    bool exact = true;
+    const bool by_warp = c > kFinSerial * (uint32_t)per;
+    if (!by_warp) sum_entries(gpts, gcovs, o, c, part, per, hi, lo, exact);
+    for (int d = 1; d < per; d <<= 1) add_lane(hi, lo, exact, d);
+    for (uint32_t todo = __ballot_sync(0xFFFFFFFFu, mine && by_warp); todo; todo &= todo - 1u) {
+      const int b = __ffs(todo) - 1;  // the whole warp sums the list of lane b
+      const uint32_t ob = __shfl_sync(0xFFFFFFFFu, o, b), cb = __shfl_sync(0xFFFFFFFFu, c, b);
+      float h[9], l[9];
+      bool ex = true;
+#pragma unroll
+      for (int k = 0; k < 9; ++k) h[k] = l[k] = 0.0f;
+      sum_entries(gpts, gcovs, ob, cb, lane, 32u, h, l, ex);
+#pragma unroll 1
+      for (int d = 1; d < 32; d <<= 1) add_lane(h, l, ex, d);
+      if (lane == b) {
+#pragma unroll
+        for (int k = 0; k < 9; ++k) {
+          hi[k] = h[k];
+          lo[k] = l[k];
+        }
+        exact = ex;
+      }
+    }
+    if (mine) {
+      write_record(v, o, c, hi, lo, exact, gpts, gcovs, recs, q);
+      insert_lookup(v, vkeys[v], c, q, map_of_rank(vbase, n_maps, r), slot_base, vmask, max_probe,
+                    vslots, lslot_of, status);
+    }
+    __syncthreads();  // the stage is reused by the next ranks
   }
 }
 
@@ -980,6 +1126,7 @@ int size_lookup_tables(MapSet* s, cudaStream_t st) {
     total += (int64_t)c;
   }
   s->vslot_base[s->n_maps] = total;
+  s->avg_list = s->n_total / std::max<int64_t>(1, (int64_t)vb[(size_t)s->n_maps]);
   if (total >= (int64_t)0xFFFFFFFFll)
     return set_error(VGICP_ERR_INVALID_ARG, "more than 2^32-1 lookup slots in one batch");
   cudaError_t e = device_malloc(&s->d_vblock, sizeof(VSlot) * (size_t)total, nullptr, false);
@@ -1098,7 +1245,11 @@ int launch_build(MapSet* s, const float* points, const float* covs, cudaStream_t
                                                              s->d_vslots, s->d_vmask,
                                                              was_built ? 0 : 1);
   // sums, records, grouped clouds and the lookup tables
-  finalize_kernel<<<g, kFinThreads, 0, st>>>(
+  // large sets of short lists (the first build's average) keep the kernel that sorts
+  // them a thread per voxel (figures at finalize_long_kernel)
+  const auto finalize =
+      s->avg_list > 10 || n < 500000 ? finalize_long_kernel : finalize_kernel;
+  finalize<<<g, kFinThreads, 0, st>>>(
       n, s->d_num_voxels, s->d_num_valid, points, covs, vorder, s->d_goff, s->d_plist, s->d_recs,
       s->d_gpts, s->d_gcovs, s->d_vkeys, s->n_maps, s->d_vbase, s->d_vslot_base, s->d_vmask,
       s->max_probe, s->d_vslots, s->d_lslot_of, s->d_status);

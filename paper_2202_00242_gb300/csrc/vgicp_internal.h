@@ -70,6 +70,7 @@ struct MapSet {
   // kept from one build to the next: the lookup-table slot each voxel occupies,
   // so a rebuild empties just those (every other slot is empty already)
   uint32_t* d_lslot_of = nullptr; // n_total: lookup-table slot of each voxel (or kNoSlot)
+  int64_t avg_list = 0;           // points per voxel of the first build (picks a kernel)
   bool built = false;             // a build has run: the lookup tables hold only its
                                   // voxels and the build table is empty
   float* d_gpts = nullptr;        // n_total x 3: the clouds grouped by voxel, voxels in
