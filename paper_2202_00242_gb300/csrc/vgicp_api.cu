@@ -504,8 +504,7 @@ int vgicp_linearize(const vgicp_map* map, const float* src_points, const float* 
   int item = opts && opts->tile > 0 ? opts->tile : 0;
   if (item == 0) {
     // spread one factor over the persistent grid, 256..16K points per item
-    const int64_t target_items =
-        linearize_grid(neighbours, opts && opts->variant ? opts->variant : default_variant());
+    const int64_t target_items = single_factor_items();
     int64_t t = (n_src + target_items - 1) / std::max<int64_t>(target_items, 1);
     t = std::max<int64_t>(256, std::min<int64_t>(default_item_size(), (t + 255) / 256 * 256));
     item = (int)t;
@@ -781,8 +780,7 @@ extern "C" int vgicp_linearize_noalloc(const vgicp_map* map, const float* src_po
     return set_error(VGICP_ERR_INVALID_ARG, "variant must be 0, 1, 2 or 3");
   int item = opts && opts->tile > 0 ? opts->tile : 0;
   if (item == 0) {
-    const int64_t target_items =
-        linearize_grid(neighbours, opts && opts->variant ? opts->variant : default_variant());
+    const int64_t target_items = single_factor_items();
     int64_t t = (n_src + target_items - 1) / std::max<int64_t>(target_items, 1);
     t = std::max<int64_t>(256, std::min<int64_t>(default_item_size(), (t + 255) / 256 * 256));
     item = (int)t;

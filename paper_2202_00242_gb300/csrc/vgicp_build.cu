@@ -228,8 +228,6 @@ __device__ __forceinline__ void insert_lookup(uint32_t v, unsigned long long key
   sl.cov[3] = l11;
   sl.cov[4] = l21;
   sl.cov[5] = l22;
-  sl.pad1[0] = 0.0f;
-  sl.pad1[1] = 0.0f;
 }
 
 // Per-voxel sums and the grouped cloud.  A CTA takes 128 consecutive ranks,

@@ -34,13 +34,15 @@ constexpr uint32_t kNoSlot = 0xFFFFFFFFu;
 //   r2 = (C'yz, C'zz, 0, 0)
 constexpr int kRecordF4 = 3;
 
-// Lookup table slot with the voxel Gaussian inline (64 B, 64-B aligned): a
-// lookup is two independent 256-bit loads; a probe that needs only the key and
-// the spill flag reads the first 16 B.
-//   bytes  0..15: key (u64), spill (u32), vid (u32)
-//   bytes 16..31: count (u32), mu' (3 x f32)
-//   bytes 32..63: L, the Cholesky factor of C' (6 x f32: l00 l10 l20 l11 l21
-//                 l22), pad
+// Lookup table slot with the voxel Gaussian inline (64 B, 64-B aligned): a lookup
+// is two independent loads, of 32 and 16 B, all of which it uses; a probe that needs
+// only the key and the spill flag reads the first 16 B.
+//   bytes  0..11: key (u64), spill (u32)
+//   bytes 12..47: mu' (3 x f32), then L, the Cholesky factor of C' (6 x f32: l00 l10
+//                 l20 l11 l21 l22)
+//   bytes 48..55: vid, count (u32), not read by lookups
+// (With vid and count among the first 32 B, a lookup loaded 64 B into 16 registers;
+// now 48 B into 12, which lets four CTAs of the linearization share an SM.)
 // Linear probing from the key's home slot h.  spill (of slot h) is nonzero iff
 // some key whose home is h lies further along the probe sequence, so a lookup
 // whose home slot holds another key and has spill == 0 is a miss after one
@@ -55,15 +57,16 @@ constexpr uint32_t kLookupLoad = VGICP_LOOKUP_LOAD;
 struct __align__(64) VSlot {
   unsigned long long key;
   uint32_t spill;
-  uint32_t vid;
-  uint32_t count;
   float mu[3];
   float cov[6];
-  float pad1[2];
+  uint32_t vid;
+  uint32_t count;
+  uint32_t pad[2];
 };
 static_assert(sizeof(VSlot) == 64, "VSlot is 64 B");
-// 32-bit words of the first half as loaded: key 0..1, then these
-constexpr int kSlotSpill = 2, kSlotVid = 3, kSlotMu = 5;
+// 32-bit words of the first half as loaded: key 0..1, then these (l00, l10 are words
+// 6 and 7)
+constexpr int kSlotSpill = 2, kSlotMu = 3, kSlotL = 6;
 
 // Per-map descriptor read by the linearize kernels.
 struct MapDesc {

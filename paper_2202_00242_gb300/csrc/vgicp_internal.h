@@ -143,7 +143,8 @@ int arm_wait_test(int32_t tile, int64_t limit_ns);
 
 // Points per work item and the persistent grid the linearize kernel uses.
 int default_item_size();
-int linearize_grid(int neighbours, int variant);
+int single_factor_items();
+int linearize_grid(int neighbours, int variant, int mode);
 int default_variant();
 
 // Sum each pair's partials over its items [span[p].x, span[p].y) in order and

@@ -56,7 +56,7 @@ struct Pose32 {
 };
 
 // floor(q_a / r) with q = R64 mu + t64 in binary64 (the rare near-face path).
-__device__ __noinline__ int axis_key_f64(const PairDesc* pd, const MapDesc& md, int a, float x,
+__device__ __forceinline__ int axis_key_f64(const PairDesc* pd, const MapDesc& md, int a, float x,
                                          float y, float z) {
   double s = __dmul_rn(pd->R64[3 * a + 0], (double)x);
   s = __dadd_rn(s, __dmul_rn(pd->R64[3 * a + 1], (double)y));
@@ -94,36 +94,35 @@ __device__ __forceinline__ void source_key(const Pose32& P, const PairDesc* pd, 
   }
 }
 
-// Two independent 256-bit loads: one probe of a 64-B lookup slot.
-#ifndef VGICP_LD_FLAVOR
-#define VGICP_LD_FLAVOR 0
-#endif
 __device__ __forceinline__ void ld_v8(const void* p, uint64_t policy, uint32_t (&w)[8]) {
-#if VGICP_LD_FLAVOR == 0
   asm("ld.global.nc.L2::cache_hint.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8], %9;"
       : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]), "=r"(w[4]), "=r"(w[5]), "=r"(w[6]),
         "=r"(w[7])
       : "l"(p), "l"(policy));
-#elif VGICP_LD_FLAVOR == 1
-  asm("ld.global.cg.L2::cache_hint.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8], %9;"
-      : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]), "=r"(w[4]), "=r"(w[5]), "=r"(w[6]),
-        "=r"(w[7])
-      : "l"(p), "l"(policy));
-#else
-  asm("ld.global.L2::cache_hint.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8], %9;"
-      : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]), "=r"(w[4]), "=r"(w[5]), "=r"(w[6]),
-        "=r"(w[7])
-      : "l"(p), "l"(policy));
-#endif
 }
 __device__ __forceinline__ unsigned long long slot_key(const uint32_t (&a)[8]) {
   return (unsigned long long)a[0] | ((unsigned long long)a[1] << 32);
 }
-// A slot's first 16 B: key (words 0, 1), spill flag, vid.
 __device__ __forceinline__ void ld_v4(const void* p, uint64_t policy, uint32_t (&w)[4]) {
   asm("ld.global.nc.L2::cache_hint.v4.b32 {%0, %1, %2, %3}, [%4], %5;"
       : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3])
       : "l"(p), "l"(policy));
+}
+// One probe of a lookup slot: two independent loads (a: key, spill, mu', l00, l10; b:
+// l20, l11, l21, l22).
+__device__ __forceinline__ void ld_slot(const VSlot* t, uint64_t policy, uint32_t (&a)[8],
+                                        uint32_t (&b)[4]) {
+  ld_v8(t, policy, a);
+  ld_v4(reinterpret_cast<const char*>(t) + 32, policy, b);
+}
+// The slot's Gaussian: r0 = (mu', -), r1 = (l00, l10, l20, l11), r2 = (l21, l22, -, -).
+__device__ __forceinline__ void slot_gaussian(const uint32_t (&a)[8], const uint32_t (&b)[4],
+                                              float4& r0, float4& r1, float4& r2) {
+  r0 = make_float4(__uint_as_float(a[kSlotMu]), __uint_as_float(a[kSlotMu + 1]),
+                   __uint_as_float(a[kSlotMu + 2]), 0.f);
+  r1 = make_float4(__uint_as_float(a[kSlotL]), __uint_as_float(a[kSlotL + 1]),
+                   __uint_as_float(b[0]), __uint_as_float(b[1]));
+  r2 = make_float4(__uint_as_float(b[2]), __uint_as_float(b[3]), 0.f, 0.f);
 }
 __device__ __forceinline__ uint64_t policy_evict_last_l() {
   uint64_t p;
@@ -131,31 +130,26 @@ __device__ __forceinline__ uint64_t policy_evict_last_l() {
   return p;
 }
 
-// Lookup of key (kx, ky, kz) in a map's inline table; on a hit returns the
-// global voxel id and the voxel Gaussian as r0 = (mu', -), r1, r2 (record layout).
-__device__ __forceinline__ int lookup(const MapDesc& md, uint32_t mask, int kx, int ky, int kz,
-                                      uint64_t pol, float4& r0, float4& r1, float4& r2) {
-  if (!key_in_range(kx) || !key_in_range(ky) || !key_in_range(kz)) return -1;
+// Lookup of key (kx, ky, kz) in a map's inline table: whether the voxel exists; on a
+// hit also its slot and Gaussian.
+__device__ __forceinline__ bool lookup(const MapDesc& md, uint32_t mask, int kx, int ky, int kz,
+                                       uint64_t pol, uint32_t& h, float4& r0, float4& r1,
+                                       float4& r2) {
+  if (!key_in_range(kx) || !key_in_range(ky) || !key_in_range(kz)) return false;
   const unsigned long long key = pack_key(kx, ky, kz);
-  uint32_t h = hash_key(kx, ky, kz) & mask;
+  h = hash_key(kx, ky, kz) & mask;
   for (int p = 0; p < md.max_probe; ++p) {
-    uint32_t a[8], b[8];
-    const VSlot* t = md.vslots + h;
-    ld_v8(t, pol, a);
-    ld_v8(reinterpret_cast<const char*>(t) + 32, pol, b);
+    uint32_t a[8], b[4];
+    ld_slot(md.vslots + h, pol, a, b);
     const unsigned long long k = slot_key(a);
     if (k == key) {
-      r0 = make_float4(__uint_as_float(a[kSlotMu]), __uint_as_float(a[kSlotMu + 1]),
-                       __uint_as_float(a[kSlotMu + 2]), 0.f);
-      r1 = make_float4(__uint_as_float(b[0]), __uint_as_float(b[1]), __uint_as_float(b[2]),
-                       __uint_as_float(b[3]));
-      r2 = make_float4(__uint_as_float(b[4]), __uint_as_float(b[5]), 0.f, 0.f);
-      return (int)a[kSlotVid];
+      slot_gaussian(a, b, r0, r1, r2);
+      return true;
     }
-    if (k == kEmptyKey || (p == 0 && a[kSlotSpill] == 0u)) return -1;  // empty, or nothing spilled
+    if (k == kEmptyKey || (p == 0 && a[kSlotSpill] == 0u)) return false;  // empty, or nothing spilled
     h = (h + 1) & mask;
   }
-  return -1;
+  return false;
 }
 
 // Accumulator layout (float):
@@ -559,7 +553,7 @@ __global__ void __launch_bounds__(kThreads, VGICP_MIN_BLOCKS) linearize_tma_kern
     bool live[kPtsPerLane];
     unsigned long long key[kPtsPerLane];
     uint32_t h[kPtsPerLane];
-    uint32_t sa[kPtsPerLane][8], sb[kPtsPerLane][8];
+    uint32_t sa[kPtsPerLane][8], sb[kPtsPerLane][4];
 #pragma unroll
     for (int k = 0; k < kPtsPerLane; ++k) {
       idx[k] = warp * kWarpPts + k * 32 + lane;
@@ -576,8 +570,7 @@ __global__ void __launch_bounds__(kThreads, VGICP_MIN_BLOCKS) linearize_tma_kern
       key[k] = live[k] ? pack_key(kx[k], ky[k], kz[k]) : kEmptyKey;
       h[k] = hash_key(kx[k], ky[k], kz[k]) & mask;
       if (live[k]) {
-        ld_v8(md.vslots + h[k], map_pol, sa[k]);
-        ld_v8(reinterpret_cast<const char*>(md.vslots + h[k]) + 32, map_pol, sb[k]);
+        ld_slot(md.vslots + h[k], map_pol, sa[k], sb[k]);
       } else {
         sa[k][0] = sa[k][1] = 0xFFFFFFFFu;
       }
@@ -594,17 +587,12 @@ __global__ void __launch_bounds__(kThreads, VGICP_MIN_BLOCKS) linearize_tma_kern
                         p < md.max_probe;
              ++p) {
           hh = (hh + 1) & mask;
-          ld_v8(md.vslots + hh, map_pol, sa[k]);
-          ld_v8(reinterpret_cast<const char*>(md.vslots + hh) + 32, map_pol, sb[k]);
+          ld_slot(md.vslots + hh, map_pol, sa[k], sb[k]);
           t = slot_key(sa[k]);
         }
         if (t == key[k]) {
-          vid[k] = (int)sa[k][kSlotVid];
-          r0[k] = make_float4(__uint_as_float(sa[k][kSlotMu]), __uint_as_float(sa[k][kSlotMu + 1]),
-                              __uint_as_float(sa[k][kSlotMu + 2]), 0.f);
-          r1[k] = make_float4(__uint_as_float(sb[k][0]), __uint_as_float(sb[k][1]),
-                              __uint_as_float(sb[k][2]), __uint_as_float(sb[k][3]));
-          r2[k] = make_float4(__uint_as_float(sb[k][4]), __uint_as_float(sb[k][5]), 0.f, 0.f);
+          vid[k] = L.corr_out ? (int)__ldg(&md.vslots[hh].vid) : 0;
+          slot_gaussian(sa[k], sb[k], r0[k], r1[k], r2[k]);
         }
       }
       if (idx[k] < d.n && (L.corr_out || L.qkey_out)) {
@@ -740,13 +728,9 @@ __device__ __forceinline__ void term(float* acc, const Pose32& P, float x, float
 // items.  Occupancy is what hides the DRAM latency of the stream and the L2
 // latency of the lookup here, so the kernel keeps its registers for the 28
 // accumulators and the term arithmetic: the constants of the current work item
-// (pose, map and source descriptors) sit in shared memory and are re-read
-// (volatile) in every iteration instead of living in registers across the
-// point loop.
+// (pose, map and source descriptors) live in uniform registers across the point
+// loop, one per warp instead of one per lane.
 // ---------------------------------------------------------------------------
-#ifndef VGICP_SIMPLE_MIN_BLOCKS
-#define VGICP_SIMPLE_MIN_BLOCKS 3
-#endif
 
 struct __align__(16) ItemConst {
   float R[9];
@@ -774,8 +758,39 @@ __device__ __forceinline__ void lds_2ptr(const void* p, uint64_t& a, uint64_t& b
                : "r"((uint32_t)__cvta_generic_to_shared(p)));
 }
 
+// A value that is the same in all lanes of the (whole) warp, through a reduction
+// whose result the compiler knows to be uniform: it then lives in a uniform register
+// instead of one register per lane.
+__device__ __forceinline__ uint32_t uniform(uint32_t v) { return __reduce_or_sync(0xFFFFFFFFu, v); }
+__device__ __forceinline__ float uniform(float v) {
+  return __uint_as_float(uniform(__float_as_uint(v)));
+}
+template <typename T>
+__device__ __forceinline__ T* uniform(T* p) {
+  const uint64_t v = reinterpret_cast<uint64_t>(p);
+  return reinterpret_cast<T*>((uint64_t)uniform((uint32_t)v) |
+                              ((uint64_t)uniform((uint32_t)(v >> 32)) << 32));
+}
+
+__device__ __forceinline__ MapDesc md_of_item(MapDesc md, double r) {
+  md.r = r;
+  return md;
+}
+
+// CTAs per SM.  The linearization, the cost and the gradients fit four (64
+// registers) with the item's constants in uniform registers, slots of 12 words and the
+// key without conversions; the overlap count fits eight.  27 neighbours are slower
+// with more CTAs (the L1 holds less of the tables).  3 CTAs, constants re-read from
+// shared memory, before: global map 2.85 -> 2.51 ms, 1,000 factors of unsorted clouds
+// 812 -> 794 us, cost and gradient of 256 factors 336 -> 244 us, overlap of 3,540
+// pairs 1,096 -> 691 us (four CTAs 820).  Three CTAs with the new code 2.82 ms; five
+// spill (3.6 ms).
+__host__ __device__ constexpr int simple_ctas(int neigh, int mode) {
+  return neigh == 27 ? 3 : mode == 4 ? 8 : 4;
+}
+
 template <int NEIGH, int MODE, bool DBG>
-__global__ void __launch_bounds__(kSimpleThreads, VGICP_SIMPLE_MIN_BLOCKS)
+__global__ void __launch_bounds__(kSimpleThreads, simple_ctas(NEIGH, MODE))
     linearize_simple_kernel(const __grid_constant__ LinLaunch L) {
   __shared__ float red[kSimpleThreads / 32][kAcc];
   // 27 neighbours: each thread's hits (slot offsets) of its current point
@@ -819,128 +834,135 @@ __global__ void __launch_bounds__(kSimpleThreads, VGICP_SIMPLE_MIN_BLOCKS)
 #pragma unroll
     for (int k = 0; k < kAcc; ++k) acc[k] = 0.0f;
 
-    for (int p = begin + threadIdx.x; p < end; p += kSimpleThreads) {
-      const float4 g0 = lds_f4(&ic.R[0]), g1 = lds_f4(&ic.R[4]), g2 = lds_f4(&ic.R[8]);
-      const float4 g3 = lds_f4(&ic.tmax);
-      uint64_t vs, ps, cs, pds;
-      lds_2ptr(&ic.vslots, vs, ps);
-      lds_2ptr(&ic.covs, cs, pds);
-      Pose32 P;
-      P.R[0] = g0.x; P.R[1] = g0.y; P.R[2] = g0.z; P.R[3] = g0.w;
-      P.R[4] = g1.x; P.R[5] = g1.y; P.R[6] = g1.z; P.R[7] = g1.w;
-      P.R[8] = g2.x;
-      P.t[0] = g2.y; P.t[1] = g2.z; P.t[2] = g2.w;
-      P.tmax = g3.x;
-      MapDesc md;
-      md.vslots = reinterpret_cast<const VSlot*>(vs);
-      md.inv_r = g3.y;
-      md.margin_scale = g3.z;
-      const uint32_t mask = __float_as_uint(g3.w);
-      const PairDesc* pd = reinterpret_cast<const PairDesc*>(pds);
+    // the item's constants in uniform registers
+    Pose32 P;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) P.R[k] = uniform(ic.R[k]);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) P.t[k] = uniform(ic.t[k]);
+    P.tmax = uniform(ic.tmax);
+    MapDesc md;
+    md.inv_r = uniform(ic.inv_r);
+    md.margin_scale = uniform(ic.margin_scale);
+    md.vslots = uniform(ic.vslots);
+    const uint32_t mask = uniform(ic.mask);
+    // 32-bit offsets from uniform bases, 2^26 points (a whole number of rounds) at a time
+    for (int64_t b0 = begin; b0 < end; b0 += 1 << 26) {
+      const char* const pts = uniform(reinterpret_cast<const char*>(ic.pts + 3 * b0));
+      const char* const covs = uniform(reinterpret_cast<const char*>(ic.covs + 6 * b0));
+      const uint32_t n_here = uniform((uint32_t)min((int64_t)1 << 26, end - b0));
 
-      const float* pt = reinterpret_cast<const float*>(ps) + 3 * (int64_t)p;
-      const float x = __ldg(pt + 0), y = __ldg(pt + 1), z = __ldg(pt + 2);
-      const float2* cv = reinterpret_cast<const float2*>(reinterpret_cast<const float*>(cs) +
-                                                         6 * (int64_t)p);
-      const float2 c01 = __ldg(cv + 0), c23 = __ldg(cv + 1), c45 = __ldg(cv + 2);
-      const float c[6] = {c01.x, c01.y, c23.x, c23.y, c45.x, c45.y};
-      const float qx = fmaf(P.R[0], x, fmaf(P.R[1], y, fmaf(P.R[2], z, P.t[0])));
-      const float qy = fmaf(P.R[3], x, fmaf(P.R[4], y, fmaf(P.R[5], z, P.t[1])));
-      const float qz = fmaf(P.R[6], x, fmaf(P.R[7], y, fmaf(P.R[8], z, P.t[2])));
-      int kx, ky, kz;
-      {
-        // the binary64 fallback reads r from shared memory only when taken
-        const float S = fabsf(x) + fabsf(y) + fabsf(z) + P.tmax;
-        const float m = fmaf(S, md.margin_scale, 1.1920928955078125e-7f);
-        const float yx = qx * md.inv_r, yy = qy * md.inv_r, yz = qz * md.inv_r;
-        const float fx = floorf(yx), fy = floorf(yy), fz = floorf(yz);
-        const float rx = yx - fx, ry = yy - fy, rz = yz - fz;
-        const bool ax = (rx < m) | (rx > 1.0f - m);
-        const bool ay = (ry < m) | (ry > 1.0f - m);
-        const bool az = (rz < m) | (rz > 1.0f - m);
-        kx = clamp_to_int(fx);
-        ky = clamp_to_int(fy);
-        kz = clamp_to_int(fz);
-        if (ax | ay | az) {
-          MapDesc mr;
-          mr.r = ic.r;
-          if (ax) kx = axis_key_f64(pd, mr, 0, x, y, z);
-          if (ay) ky = axis_key_f64(pd, mr, 1, x, y, z);
-          if (az) kz = axis_key_f64(pd, mr, 2, x, y, z);
-        }
-      }
-      if (DBG && L.qkey_out) {
-        L.qkey_out[3 * (int64_t)p + 0] = kx;
-        L.qkey_out[3 * (int64_t)p + 1] = ky;
-        L.qkey_out[3 * (int64_t)p + 2] = kz;
-      }
-      md.max_probe = ic.max_probe;
-      if (NEIGH == 1) {
-        float4 a0, a1, a2;
-        const int vid = lookup(md, mask, kx, ky, kz, pol, a0, a1, a2);
-        if (DBG && L.corr_out) L.corr_out[p] = vid < 0 ? -1 : (int)((uint32_t)vid - vbase);
-        if (vid >= 0) term<MODE>(acc, P, x, y, z, c, qx, qy, qz, a0, a1, a2);
-        continue;
-      }
-      if (DBG && L.corr_out) {
-        float4 a0, a1, a2;
-        const int own = lookup(md, mask, kx, ky, kz, pol, a0, a1, a2);
-        L.corr_out[p] = own < 0 ? -1 : (int)((uint32_t)own - vbase);
-      }
-      // the 27 probes first, hits recorded; then the terms, hit by hit, so a
-      // warp evaluates a term while most of its lanes still have one.  The
-      // probes go a row of three neighbours at a time, their home slots' first
-      // 16 B (key, spill flag) loaded together; a miss whose home slot holds
-      // another key with its spill flag set probes on
-      int nh = 0;
-      for (int dz = -1; dz <= 1; ++dz)
-        for (int dy = -1; dy <= 1; ++dy) {
-          const int yy = ky + dy, zz = kz + dz;
-          const bool row_ok = key_in_range(yy) && key_in_range(zz);
-          uint32_t A[3][4];
-          uint32_t hh[3];
-#pragma unroll
-          for (int j = 0; j < 3; ++j) {
-            hh[j] = hash_key(kx + j - 1, yy, zz) & mask;
-            ld_v4(md.vslots + hh[j], pol, A[j]);
+      for (uint32_t i = threadIdx.x; i < n_here; i += kSimpleThreads) {
+        const float* pt = reinterpret_cast<const float*>(pts + 12u * i);
+        const float2* cv = reinterpret_cast<const float2*>(covs + 24u * i);
+        const float x = __ldg(pt + 0), y = __ldg(pt + 1), z = __ldg(pt + 2);
+        const float2 c01 = __ldg(cv + 0), c23 = __ldg(cv + 1), c45 = __ldg(cv + 2);
+        const float c[6] = {c01.x, c01.y, c23.x, c23.y, c45.x, c45.y};
+        const float qx = fmaf(P.R[0], x, fmaf(P.R[1], y, fmaf(P.R[2], z, P.t[0])));
+        const float qy = fmaf(P.R[3], x, fmaf(P.R[4], y, fmaf(P.R[5], z, P.t[1])));
+        const float qz = fmaf(P.R[6], x, fmaf(P.R[7], y, fmaf(P.R[8], z, P.t[2])));
+        // Exact key.  y = q / r is split into the nearest integer n and f = y - n (exact)
+        // by adding and subtracting 1.5 * 2^23; floor(y) = n - (f < 0), and a face is
+        // near when |f| is below the margin of source_key.  |y| >= 2^22 (and NaN) lies
+        // outside the key range.
+        int kx, ky, kz;
+        {
+          const float m = fmaf(fabsf(x) + fabsf(y) + fabsf(z) + P.tmax, md.margin_scale,
+                               1.1920928955078125e-7f);
+          const float yx = qx * md.inv_r, yy = qy * md.inv_r, yz = qz * md.inv_r;
+          constexpr float kMagic = 12582912.0f;
+          constexpr int kMagicBits = 0x4B400000;
+          const float nx = yx + kMagic, ny = yy + kMagic, nz = yz + kMagic;
+          const float fx = yx - (nx - kMagic), fy = yy - (ny - kMagic), fz = yz - (nz - kMagic);
+          kx = __float_as_int(nx) - kMagicBits + (__float_as_int(fx) >> 31);
+          ky = __float_as_int(ny) - kMagicBits + (__float_as_int(fy) >> 31);
+          kz = __float_as_int(nz) - kMagicBits + (__float_as_int(fz) >> 31);
+          const bool inside =
+              fabsf(yx) < 4194304.0f && fabsf(yy) < 4194304.0f && fabsf(yz) < 4194304.0f;
+          const bool ax = fabsf(fx) < m, ay = fabsf(fy) < m, az = fabsf(fz) < m;
+          if (inside && (ax | ay | az)) {  // the binary64 path reads r from shared memory
+            MapDesc mr;
+            mr.r = ic.r;
+            if (ax) kx = axis_key_f64(ic.pd, mr, 0, x, y, z);
+            if (ay) ky = axis_key_f64(ic.pd, mr, 1, x, y, z);
+            if (az) kz = axis_key_f64(ic.pd, mr, 2, x, y, z);
           }
+          if (!inside) {
+            if (DBG) source_key(P, ic.pd, md_of_item(md, ic.r), x, y, z, qx, qy, qz, kx, ky, kz);
+            else kx = 2 * kKeyMin;  // no neighbour is in range either
+          }
+        }
+        if (DBG && L.qkey_out) {
+          L.qkey_out[3 * (b0 + i) + 0] = kx;
+          L.qkey_out[3 * (b0 + i) + 1] = ky;
+          L.qkey_out[3 * (b0 + i) + 2] = kz;
+        }
+        md.max_probe = ic.max_probe;
+        if (NEIGH == 1) {
+          float4 a0, a1, a2;
+          uint32_t h = 0u;
+          const bool hit = lookup(md, mask, kx, ky, kz, pol, h, a0, a1, a2);
+          if (DBG && L.corr_out) L.corr_out[b0 + i] = hit ? (int)(md.vslots[h].vid - vbase) : -1;
+          if (hit) term<MODE>(acc, P, x, y, z, c, qx, qy, qz, a0, a1, a2);
+          continue;
+        }
+        if (DBG && L.corr_out) {
+          float4 a0, a1, a2;
+          uint32_t h = 0u;
+          L.corr_out[b0 + i] = lookup(md, mask, kx, ky, kz, pol, h, a0, a1, a2)
+                              ? (int)(md.vslots[h].vid - vbase)
+                              : -1;
+        }
+        // the 27 probes first, hits recorded; then the terms, hit by hit, so a
+        // warp evaluates a term while most of its lanes still have one.  The
+        // probes go a row of three neighbours at a time, their home slots' first
+        // 16 B (key, spill flag) loaded together; a miss whose home slot holds
+        // another key with its spill flag set probes on
+        int nh = 0;
+        for (int dz = -1; dz <= 1; ++dz)
+          for (int dy = -1; dy <= 1; ++dy) {
+            const int yy = ky + dy, zz = kz + dz;
+            const bool row_ok = key_in_range(yy) && key_in_range(zz);
+            uint32_t A[3][4];
+            uint32_t hh[3];
 #pragma unroll
-          for (int j = 0; j < 3; ++j) {
-            const int xx = kx + j - 1;
-            if (!row_ok || !key_in_range(xx)) continue;
-            const unsigned long long key = pack_key(xx, yy, zz);
-            const unsigned long long k0 =
-                (unsigned long long)A[j][0] | ((unsigned long long)A[j][1] << 32);
-            int hs = -1;
-            if (k0 == key) {
-              hs = (int)hh[j];
-            } else if (k0 != kEmptyKey && A[j][kSlotSpill] != 0u) {
-              uint32_t h = (hh[j] + 1) & mask;  // spilled keys: probe on
-              for (int q = 1; q < md.max_probe; ++q) {
-                uint32_t a[4];
-                ld_v4(md.vslots + h, pol, a);
-                const unsigned long long k =
-                    (unsigned long long)a[0] | ((unsigned long long)a[1] << 32);
-                if (k == key) { hs = (int)h; break; }
-                if (k == kEmptyKey) break;
-                h = (h + 1) & mask;
-              }
+            for (int j = 0; j < 3; ++j) {
+              hh[j] = hash_key(kx + j - 1, yy, zz) & mask;
+              ld_v4(md.vslots + hh[j], pol, A[j]);
             }
-            if (hs >= 0) hits[27 * threadIdx.x + nh++] = (uint32_t)hs;
+#pragma unroll
+            for (int j = 0; j < 3; ++j) {
+              const int xx = kx + j - 1;
+              if (!row_ok || !key_in_range(xx)) continue;
+              const unsigned long long key = pack_key(xx, yy, zz);
+              const unsigned long long k0 =
+                  (unsigned long long)A[j][0] | ((unsigned long long)A[j][1] << 32);
+              int hs = -1;
+              if (k0 == key) {
+                hs = (int)hh[j];
+              } else if (k0 != kEmptyKey && A[j][kSlotSpill] != 0u) {
+                uint32_t h = (hh[j] + 1) & mask;  // spilled keys: probe on
+                for (int q = 1; q < md.max_probe; ++q) {
+                  uint32_t a[4];
+                  ld_v4(md.vslots + h, pol, a);
+                  const unsigned long long k =
+                      (unsigned long long)a[0] | ((unsigned long long)a[1] << 32);
+                  if (k == key) { hs = (int)h; break; }
+                  if (k == kEmptyKey) break;
+                  h = (h + 1) & mask;
+                }
+              }
+              if (hs >= 0) hits[27 * threadIdx.x + nh++] = (uint32_t)hs;
+            }
           }
+        for (int k = 0; k < nh; ++k) {
+          const VSlot* t = md.vslots + hits[27 * threadIdx.x + k];
+          uint32_t a[8], b[4];
+          float4 a0, a1, a2;
+          ld_slot(t, pol, a, b);
+          slot_gaussian(a, b, a0, a1, a2);
+          term<MODE>(acc, P, x, y, z, c, qx, qy, qz, a0, a1, a2);
         }
-      for (int k = 0; k < nh; ++k) {
-        const VSlot* t = md.vslots + hits[27 * threadIdx.x + k];
-        // count and mu' (bytes 16..31), then L (bytes 32..63)
-        uint32_t a[4], b[8];
-        ld_v4(reinterpret_cast<const char*>(t) + 16, pol, a);
-        ld_v8(reinterpret_cast<const char*>(t) + 32, pol, b);
-        const float4 a0 = make_float4(__uint_as_float(a[1]), __uint_as_float(a[2]),
-                                      __uint_as_float(a[3]), 0.f);
-        const float4 a1 = make_float4(__uint_as_float(b[0]), __uint_as_float(b[1]),
-                                      __uint_as_float(b[2]), __uint_as_float(b[3]));
-        const float4 a2 = make_float4(__uint_as_float(b[4]), __uint_as_float(b[5]), 0.f, 0.f);
-        term<MODE>(acc, P, x, y, z, c, qx, qy, qz, a0, a1, a2);
       }
     }
 
@@ -1084,8 +1106,8 @@ __global__ void __launch_bounds__(kThreads, VGICP_COMPACT_MIN_BLOCKS)
         md.vslots = reinterpret_cast<const VSlot*>(vs);
         md.max_probe = ic.max_probe;
         float4 a0;
-        const int vid = lookup(md, __float_as_uint(g3.w), kx, ky, kz, pol, a0, a1, a2);
-        hit = vid >= 0;
+        uint32_t h = 0u;
+        hit = lookup(md, __float_as_uint(g3.w), kx, ky, kz, pol, h, a0, a1, a2);
         tx = a0.x - qx;
         ty = a0.y - qy;
         tz = a0.z - qz;
@@ -1257,7 +1279,7 @@ __global__ void __cluster_dims__(kCtas, 1, 1) __launch_bounds__(kThreads, 2)
     // ---- kPer points per thread: key, first probe of each, resolve, terms ----
     float x[kPer], y[kPer], z[kPer], c[kPer][6], q[kPer][3];
     int kx[kPer], ky[kPer], kz[kPer];
-    uint32_t h[kPer], sa[kPer][8], sb[kPer][8];
+    uint32_t h[kPer], sa[kPer][8], sb[kPer][4];
     unsigned long long key[kPer];
     bool live[kPer];
 #pragma unroll
@@ -1288,8 +1310,7 @@ __global__ void __cluster_dims__(kCtas, 1, 1) __launch_bounds__(kThreads, 2)
       if (live[u]) {
         key[u] = pack_key(kx[u], ky[u], kz[u]);
         h[u] = hash_key(kx[u], ky[u], kz[u]) & mask;
-        ld_v8(md.vslots + h[u], pol, sa[u]);
-        ld_v8(reinterpret_cast<const char*>(md.vslots + h[u]) + 32, pol, sb[u]);
+        ld_slot(md.vslots + h[u], pol, sa[u], sb[u]);
       }
     }
 #pragma unroll
@@ -1301,8 +1322,7 @@ __global__ void __cluster_dims__(kCtas, 1, 1) __launch_bounds__(kThreads, 2)
                         p < md.max_probe;
              ++p) {
           h[u] = (h[u] + 1) & mask;
-          ld_v8(md.vslots + h[u], pol, sa[u]);
-          ld_v8(reinterpret_cast<const char*>(md.vslots + h[u]) + 32, pol, sb[u]);
+          ld_slot(md.vslots + h[u], pol, sa[u], sb[u]);
           t = slot_key(sa[u]);
         }
         hit = t == key[u];
@@ -1311,12 +1331,9 @@ __global__ void __cluster_dims__(kCtas, 1, 1) __launch_bounds__(kThreads, 2)
 #pragma unroll
       for (int k = 0; k < NV; ++k) v[k] = 0.0f;  // a miss adds zeros
       if (hit) {
-        const float tx = __uint_as_float(sa[u][kSlotMu]) - q[u][0];
-        const float ty = __uint_as_float(sa[u][kSlotMu + 1]) - q[u][1];
-        const float tz = __uint_as_float(sa[u][kSlotMu + 2]) - q[u][2];
-        const float4 r1 = make_float4(__uint_as_float(sb[u][0]), __uint_as_float(sb[u][1]),
-                                      __uint_as_float(sb[u][2]), __uint_as_float(sb[u][3]));
-        const float4 r2 = make_float4(__uint_as_float(sb[u][4]), __uint_as_float(sb[u][5]), 0.f, 0.f);
+        float4 r0, r1, r2;
+        slot_gaussian(sa[u], sb[u], r0, r1, r2);
+        const float tx = r0.x - q[u][0], ty = r0.y - q[u][1], tz = r0.z - q[u][2];
         const float d0 = fmaf(R[0], tx, fmaf(R[3], ty, R[6] * tz));
         const float d1 = fmaf(R[1], tx, fmaf(R[4], ty, R[7] * tz));
         const float d2 = fmaf(R[2], tx, fmaf(R[5], ty, R[8] * tz));
@@ -1562,9 +1579,14 @@ int default_item_size() { return 16384; }
 
 int default_variant() { return 1; }
 
-int linearize_grid(int neighbours, int variant) {
+// Work items a single factor is spread over (which fixes the order of its sums, so
+// it stays when a kernel's CTAs per SM change).
+int single_factor_items() { return device_sm_count() * 3; }
+
+int linearize_grid(int neighbours, int variant, int mode) {
   if (variant == 0) variant = default_variant();
-  if (neighbours == 27 || variant == 1) return device_sm_count() * VGICP_SIMPLE_MIN_BLOCKS;
+  if (neighbours == 27 || variant == 1 || mode != 0)
+    return device_sm_count() * simple_ctas(neighbours, mode);
   if (variant == 3) return device_sm_count() * VGICP_COMPACT_MIN_BLOCKS;
   return device_sm_count() * VGICP_MIN_BLOCKS;
 }
@@ -1583,7 +1605,7 @@ static bool split_items(const LinLaunch& L, int variant) {
 int launch_linearize(const LinLaunch& L, cudaStream_t st) {
   if (L.n_items <= 0) return VGICP_OK;
   const int variant = L.mode != 0 ? 1 : (L.variant ? L.variant : default_variant());
-  int grid = L.grid > 0 ? L.grid : linearize_grid(L.neighbours, variant);
+  int grid = L.grid > 0 ? L.grid : linearize_grid(L.neighbours, variant, L.mode);
   grid = std::min(grid, L.n_items);
   if (L.ev_start) VGICP_CUDA_TRY(cudaEventRecord(L.ev_start, st));
   if (split_items(L, variant)) {

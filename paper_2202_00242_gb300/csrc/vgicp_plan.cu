@@ -467,7 +467,7 @@ int vgicp_plan_info(const vgicp_plan* P, int32_t* variant, int32_t* item_points,
   if (variant) *variant = P->variant ? P->variant : default_variant();
   if (item_points) *item_points = P->item;
   if (grid)
-    *grid = P->grid ? P->grid : std::min<int64_t>(linearize_grid(P->neighbours, P->variant),
+    *grid = P->grid ? P->grid : std::min<int64_t>(linearize_grid(P->neighbours, P->variant, 0),
                                                   P->n_items);
   if (n_items) *n_items = P->n_items;
   return VGICP_OK;
