@@ -13,16 +13,25 @@
 // binary64 sums in index order).
 //
 //   insert   per point: exact key, CAS into the cloud's table, first index
-//   group    per point: sub-voxel from the first point's time; first index of
-//            each (voxel, sub) group
-//   scan     output ids in first-appearance order
-//   count, scan, scatter: the points of each output voxel, contiguous
-//   finalize per output voxel: sort its list, exact sums, means
+//   group    per point: sub-voxel from the first point's time; first index and
+//            count of each (voxel, sub) group
+//   mark     first points in a bitmap; places for the groups' point lists
+//   scatter  the points of each group, contiguous; beside it, the scan of the
+//            bitmap's words (a group's output voxel is the number of first points
+//            before its own) and the clouds' output offsets
+//   finalize per first point: exact sums of its group's list, means.  The sums are
+//            exact in any order, so the lists are not sorted (only a group whose
+//            partial sums round is, for the binary64 sum in index order)
+// Six launches, one copy in and one out: a sweep of 60,000 points is bound by their
+// latency and the host's (290 -> 215 us a call, of which the kernels take 33 us; before,
+// 14 kernels, three fills and five copies, 65 us, and a thread per voxel that sorted
+// and summed lists of thousands).
 #include <cuda_runtime.h>
 
 #include <algorithm>
 #include <cmath>
 #include <cstdint>
+#include <cstring>
 #include <string>
 #include <vector>
 
@@ -43,6 +52,14 @@ struct __align__(16) DsSlot {
   uint32_t pad;
 };
 
+// A (voxel, sub) group: G per slot, G = 2 with a time split, else 1.
+struct __align__(16) DsGroup {
+  uint32_t first;  // smallest point index
+  uint32_t count;
+  uint32_t end;    // of its list, once the scatter is done
+  uint32_t pad;
+};
+
 __device__ __forceinline__ int cloud_of(const int64_t* __restrict__ off, int32_t n, int64_t i) {
   int lo = 0, hi = n;
   while (hi - lo > 1) {
@@ -60,15 +77,10 @@ __device__ __forceinline__ void set_status(int32_t* status, int32_t code) {
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < (n); \
        i += (int64_t)gridDim.x * blockDim.x)
 
-__global__ void ds_init_kernel(DsSlot* slots, int64_t cap, uint32_t* gfirst) {
-  DS_LOOP(s, cap) {
-    DsSlot e;
-    e.key = kEmptyKey;
-    e.first = kNone;
-    e.pad = 0u;
-    slots[s] = e;
-    gfirst[2 * s] = kNone;
-    gfirst[2 * s + 1] = kNone;
+__global__ void ds_init_kernel(uint4* slots, int64_t cap, uint4* groups, int64_t n_groups) {
+  DS_LOOP(s, n_groups) {
+    if (s < cap) slots[s] = make_uint4(0xFFFFFFFFu, 0xFFFFFFFFu, kNone, 0u);
+    groups[s] = make_uint4(kNone, 0u, 0u, 0u);
   }
 }
 
@@ -114,9 +126,9 @@ __global__ void ds_insert_kernel(const float* __restrict__ pts, int64_t n,
   }
 }
 
-__global__ void ds_group_kernel(int64_t n, const float* __restrict__ times, double split,
+__global__ void ds_group_kernel(int64_t n, const float* __restrict__ times, double split, int G,
                                 const DsSlot* __restrict__ slots,
-                                const uint32_t* __restrict__ pt_slot, uint32_t* gfirst,
+                                const uint32_t* __restrict__ pt_slot, DsGroup* groups,
                                 uint32_t* __restrict__ pt_group) {
   DS_LOOP(i, n) {
     const uint32_t s = pt_slot[i];
@@ -124,69 +136,224 @@ __global__ void ds_group_kernel(int64_t n, const float* __restrict__ times, doub
       pt_group[i] = kNone;
       continue;
     }
-    uint32_t sub = 0u;
-    if (times && split > 0.0) {
+    uint32_t g = s;
+    if (G == 2) {
       const double t0 = (double)times[slots[s].first];
-      sub = fabs((double)times[i] - t0) > split ? 1u : 0u;
+      g = 2u * s + (fabs((double)times[i] - t0) > split ? 1u : 0u);
     }
-    const uint32_t g = 2u * s + sub;
-    atomicMin(&gfirst[g], (uint32_t)i);
+    atomicMin(&groups[g].first, (uint32_t)i);
+    atomicAdd(&groups[g].count, 1u);
     pt_group[i] = g;
   }
 }
 
-__global__ void ds_flags_kernel(int64_t n, const uint32_t* __restrict__ pt_group,
-                                const uint32_t* __restrict__ gfirst, uint32_t* __restrict__ flag) {
-  DS_LOOP(i, n) {
-    const uint32_t g = pt_group[i];
-    flag[i] = (g != kNone && gfirst[g] == (uint32_t)i) ? 1u : 0u;
-  }
-}
-
-__global__ void ds_assign_kernel(int64_t n, const uint32_t* __restrict__ flag,
-                                 const uint32_t* __restrict__ prefix,
-                                 const uint32_t* __restrict__ pt_group, uint32_t* __restrict__ gmap) {
-  DS_LOOP(i, n) {
-    if (flag[i]) gmap[pt_group[i]] = prefix[i];
-  }
-}
-
-__global__ void ds_count_kernel(int64_t n, const uint32_t* __restrict__ pt_group,
-                                const uint32_t* __restrict__ gmap, uint32_t* gcount,
-                                uint32_t* __restrict__ pt_out) {
-  DS_LOOP(i, n) {
-    const uint32_t g = pt_group[i];
-    if (g == kNone) {
-      pt_out[i] = kNone;
-      continue;
+// CTAs [0, n_mark): first points, one bit each (n_words words, the last one holds
+// point n's).  The others: places of the groups' lists, a range per CTA and the
+// groups' own inside it (the order of the lists does not matter).
+constexpr int kPlacePer = 4;
+__global__ void __launch_bounds__(kThreads) ds_mark_kernel(int64_t n, int64_t n_words, int n_mark,
+                                                           const uint32_t* __restrict__ pt_group,
+                                                           DsGroup* groups, int64_t n_groups,
+                                                           uint32_t* __restrict__ bitmap,
+                                                           uint32_t* cursor) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  if ((int)blockIdx.x < n_mark) {
+    const int64_t i = blockIdx.x * (int64_t)kThreads + threadIdx.x;
+    bool f = false;
+    if (i < n) {
+      const uint32_t g = pt_group[i];
+      f = g != kNone && groups[g].first == (uint32_t)i;
     }
-    const uint32_t v = gmap[g];
-    atomicAdd(gcount + v, 1u);
-    pt_out[i] = v;
+    const uint32_t b = __ballot_sync(0xFFFFFFFFu, f);
+    if (lane == 0 && (i >> 5) < n_words) bitmap[i >> 5] = b;
+    return;
+  }
+  __shared__ uint32_t warp_sum[kThreads / 32];
+  __shared__ uint32_t base;
+  const int64_t g0 = ((int64_t)blockIdx.x - n_mark) * (kThreads * kPlacePer) + threadIdx.x;
+  uint32_t cnt[kPlacePer], sum = 0u;
+#pragma unroll
+  for (int j = 0; j < kPlacePer; ++j) {
+    const int64_t g = g0 + (int64_t)j * kThreads;
+    cnt[j] = g < n_groups ? groups[g].count : 0u;
+    sum += cnt[j];
+  }
+  uint32_t inc = sum;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, inc, o);
+    if (lane >= o) inc += y;
+  }
+  if (lane == 31) warp_sum[w] = inc;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    uint32_t t = 0u;
+    for (int k = 0; k < kThreads / 32; ++k) {
+      const uint32_t x = warp_sum[k];
+      warp_sum[k] = t;
+      t += x;
+    }
+    base = t > 0u ? atomicAdd(cursor, t) : 0u;
+  }
+  __syncthreads();
+  uint32_t run = base + warp_sum[w] + inc - sum;
+#pragma unroll
+  for (int j = 0; j < kPlacePer; ++j) {
+    if (cnt[j] > 0u) groups[g0 + (int64_t)j * kThreads].end = run;  // the list's start, for now
+    run += cnt[j];
   }
 }
 
-__global__ void ds_scatter_kernel(int64_t n, const uint32_t* __restrict__ pt_out,
-                                  const uint32_t* __restrict__ goff, uint32_t* gfill,
-                                  uint32_t* __restrict__ list) {
-  DS_LOOP(i, n) {
-    const uint32_t v = pt_out[i];
-    if (v == kNone) continue;
-    list[goff[v] + atomicAdd(gfill + v, 1u)] = (uint32_t)i;
+__device__ __forceinline__ uint32_t rank_of(const uint32_t* __restrict__ bitmap,
+                                            const uint32_t* __restrict__ wscan, int64_t i) {
+  return wscan[i >> 5] + (uint32_t)__popc(bitmap[i >> 5] & ((1u << (i & 31)) - 1u));
+}
+
+__device__ __forceinline__ void scatter_point(int64_t i, const uint32_t* __restrict__ pt_group,
+                                              DsGroup* groups, uint32_t* __restrict__ list) {
+  const uint32_t g = pt_group[i];
+  if (g != kNone) list[atomicAdd(&groups[g].end, 1u)] = (uint32_t)i;
+}
+
+// CTA 0 scans the words' popcounts and writes the clouds' output offsets (and the
+// status word behind them); the others scatter the points.  For up to kScanWords
+// words, which one CTA scans while the others work.
+constexpr int64_t kScanWords = 16384;
+__global__ void __launch_bounds__(kThreads) ds_scatter_kernel(
+    int64_t n, const uint32_t* __restrict__ pt_group, DsGroup* groups, uint32_t* __restrict__ list,
+    int64_t n_words, const uint32_t* __restrict__ bitmap, uint32_t* __restrict__ wscan,
+    int32_t n_clouds, const int64_t* __restrict__ off, const int32_t* __restrict__ status,
+    uint32_t* __restrict__ oo) {
+  if (blockIdx.x > 0) {
+    const int64_t i = ((int64_t)blockIdx.x - 1) * kThreads + threadIdx.x;
+    if (i < n) scatter_point(i, pt_group, groups, list);
+    return;
+  }
+  constexpr int kPer = 8;
+  __shared__ uint32_t warp_sum[kThreads / 32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  uint32_t carry = 0u;
+  for (int64_t w0 = 0; w0 < n_words; w0 += kThreads * kPer) {
+    const int64_t a = w0 + (int64_t)threadIdx.x * kPer;
+    uint32_t c[kPer], sum = 0u;
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+      c[k] = a + k < n_words ? (uint32_t)__popc(bitmap[a + k]) : 0u;
+      sum += c[k];
+    }
+    uint32_t inc = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, inc, o);
+      if (lane >= o) inc += y;
+    }
+    if (lane == 31) warp_sum[w] = inc;
+    __syncthreads();
+    uint32_t run = carry + inc - sum;
+    for (int k = 0; k < kThreads / 32; ++k) {
+      const uint32_t x = warp_sum[k];
+      if (k < w) run += x;
+      carry += x;
+    }
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+      if (a + k < n_words) wscan[a + k] = run;
+      run += c[k];
+    }
+    __syncthreads();  // also: this CTA's words are visible to it below
+  }
+  for (int c = threadIdx.x; c <= n_clouds; c += kThreads) oo[c] = rank_of(bitmap, wscan, off[c]);
+  if (threadIdx.x == 0) oo[n_clouds + 1] = (uint32_t)*status;
+}
+
+// The same steps apart, for more words.
+__global__ void ds_popc_kernel(int64_t n_words, const uint32_t* __restrict__ bitmap,
+                               uint32_t* __restrict__ out) {
+  DS_LOOP(w, n_words) out[w] = (uint32_t)__popc(bitmap[w]);
+}
+__global__ void ds_scatter_large_kernel(int64_t n, const uint32_t* __restrict__ pt_group,
+                                        DsGroup* groups, uint32_t* __restrict__ list,
+                                        const uint32_t* __restrict__ bitmap,
+                                        const uint32_t* __restrict__ wscan, int32_t n_clouds,
+                                        const int64_t* __restrict__ off,
+                                        const int32_t* __restrict__ status,
+                                        uint32_t* __restrict__ oo) {
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (i < n) scatter_point(i, pt_group, groups, list);
+  if (i <= n_clouds) oo[i] = rank_of(bitmap, wscan, off[i]);
+  if (i == 0) oo[n_clouds + 1] = (uint32_t)*status;
+}
+
+// (hi, lo) += the same of the lane at distance `delta`, exactly (checked).
+__device__ __forceinline__ void ds_add_lane(float* hi, float* lo, bool& exact, int delta) {
+  const bool other = __shfl_xor_sync(0xFFFFFFFFu, (int)exact, delta) != 0;
+  exact = exact && other;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const float h = __shfl_xor_sync(0xFFFFFFFFu, hi[k], delta);
+    const float l = __shfl_xor_sync(0xFFFFFFFFu, lo[k], delta);
+    float t, e, u, e2, v, e3;
+    two_sum(hi[k], h, t, e);
+    two_sum(lo[k], l, u, e2);
+    two_sum(u, e, v, e3);
+    exact = exact && e2 == 0.0f && e3 == 0.0f;
+    two_sum(t, v, hi[k], lo[k]);
   }
 }
 
-__global__ void ds_finalize_kernel(int64_t n_max, const uint32_t* __restrict__ n_out,
-                                   const float* __restrict__ pts, const float* __restrict__ times,
-                                   const uint32_t* __restrict__ gcount,
-                                   const uint32_t* __restrict__ goff, uint32_t* __restrict__ list,
-                                   float* __restrict__ out_pts, float* __restrict__ out_times,
-                                   int32_t* __restrict__ out_counts) {
-  const int64_t V = min((int64_t)*n_out, n_max);
-  DS_LOOP(v, V) {
-    const uint32_t c = gcount[v];
-    uint32_t* L = list + goff[v];
-    for (uint32_t a = 1; a < c; ++a) {  // ascending point index
+// One lane per point; the lanes of first points take their group's list, lists
+// longer than kSerial the whole warp.
+constexpr uint32_t kSerial = 8;
+__global__ void __launch_bounds__(kThreads) ds_finalize_kernel(
+    int64_t n, const uint32_t* __restrict__ bitmap, const uint32_t* __restrict__ wscan,
+    const uint32_t* __restrict__ pt_group, const DsGroup* __restrict__ groups,
+    const float* __restrict__ pts, const float* __restrict__ times, uint32_t* __restrict__ list,
+    float* __restrict__ out_pts, float* __restrict__ out_times, int32_t* __restrict__ out_counts) {
+  const int64_t i = blockIdx.x * (int64_t)kThreads + threadIdx.x;
+  const int lane = threadIdx.x & 31;
+  const bool mine = i < n && ((bitmap[i >> 5] >> (i & 31)) & 1u);
+  uint32_t c = 0u, at = 0u;
+  if (mine) {
+    const uint4 g = *reinterpret_cast<const uint4*>(groups + pt_group[i]);
+    c = g.y;
+    at = g.z - g.y;
+  }
+  float hi[4] = {0.f, 0.f, 0.f, 0.f}, lo[4] = {0.f, 0.f, 0.f, 0.f};
+  bool exact = true;
+  auto add = [&](uint32_t entry, float* h, float* l, bool& ex) {
+    const int64_t j = list[entry];
+    df_add(h[0], l[0], pts[3 * j], ex);
+    df_add(h[1], l[1], pts[3 * j + 1], ex);
+    df_add(h[2], l[2], pts[3 * j + 2], ex);
+    if (times) df_add(h[3], l[3], times[j], ex);
+  };
+  if (c <= kSerial)
+    for (uint32_t a = 0; a < c; ++a) add(at + a, hi, lo, exact);
+  for (uint32_t todo = __ballot_sync(0xFFFFFFFFu, c > kSerial); todo; todo &= todo - 1u) {
+    const int b = __ffs(todo) - 1;
+    const uint32_t ab = __shfl_sync(0xFFFFFFFFu, at, b), cb = __shfl_sync(0xFFFFFFFFu, c, b);
+    float h[4] = {0.f, 0.f, 0.f, 0.f}, l[4] = {0.f, 0.f, 0.f, 0.f};
+    bool ex = true;
+    for (uint32_t a = lane; a < cb; a += 32) add(ab + a, h, l, ex);
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) ds_add_lane(h, l, ex, d);
+    if (lane == b) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        hi[k] = h[k];
+        lo[k] = l[k];
+      }
+      exact = ex;
+    }
+  }
+  if (!mine) return;
+  double s[4];
+  if (exact) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) s[k] = __dadd_rn((double)hi[k], (double)lo[k]);
+  } else {  // binary64 sums in ascending point index
+    uint32_t* L = list + at;
+    for (uint32_t a = 1; a < c; ++a) {
       const uint32_t x = L[a];
       int b = (int)a - 1;
       while (b >= 0 && L[b] > x) {
@@ -195,40 +362,21 @@ __global__ void ds_finalize_kernel(int64_t n_max, const uint32_t* __restrict__ n
       }
       L[b + 1] = x;
     }
-    float hi[4] = {0.f, 0.f, 0.f, 0.f}, lo[4] = {0.f, 0.f, 0.f, 0.f};
-    bool exact = true;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) s[k] = 0.0;
     for (uint32_t a = 0; a < c; ++a) {
       const int64_t j = L[a];
-      df_add(hi[0], lo[0], pts[3 * j], exact);
-      df_add(hi[1], lo[1], pts[3 * j + 1], exact);
-      df_add(hi[2], lo[2], pts[3 * j + 2], exact);
-      if (times) df_add(hi[3], lo[3], times[j], exact);
+#pragma unroll
+      for (int k = 0; k < 3; ++k) s[k] = __dadd_rn(s[k], (double)pts[3 * j + k]);
+      if (times) s[3] = __dadd_rn(s[3], (double)times[j]);
     }
-    double s[4];
-    if (exact) {
-      for (int k = 0; k < 4; ++k) s[k] = __dadd_rn((double)hi[k], (double)lo[k]);
-    } else {
-      for (int k = 0; k < 4; ++k) s[k] = 0.0;
-      for (uint32_t a = 0; a < c; ++a) {
-        const int64_t j = L[a];
-        for (int k = 0; k < 3; ++k) s[k] = __dadd_rn(s[k], (double)pts[3 * j + k]);
-        if (times) s[3] = __dadd_rn(s[3], (double)times[j]);
-      }
-    }
-    const double N = (double)c, y = __drcp_rn(N);
-    for (int k = 0; k < 3; ++k) out_pts[3 * v + k] = __double2float_rn(div_rn(s[k], N, y));
-    if (out_times) out_times[v] = __double2float_rn(div_rn(s[3], N, y));
-    if (out_counts) out_counts[v] = (int32_t)c;
   }
-}
-
-__global__ void ds_offsets_kernel(int32_t n_clouds, int64_t n, const int64_t* __restrict__ off,
-                                  const uint32_t* __restrict__ prefix,
-                                  const uint32_t* __restrict__ n_out, uint32_t* __restrict__ oo) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c > n_clouds) return;
-  const int64_t o = off[c];
-  oo[c] = o < n ? prefix[o] : *n_out;
+  const int64_t v = rank_of(bitmap, wscan, i);
+  const double N = (double)c, y = __drcp_rn(N);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) out_pts[3 * v + k] = __double2float_rn(div_rn(s[k], N, y));
+  if (out_times) out_times[v] = __double2float_rn(div_rn(s[3], N, y));
+  if (out_counts) out_counts[v] = (int32_t)c;
 }
 
 int grid_of(int64_t n) {
@@ -273,29 +421,35 @@ int vgicp_downsample(const float* points, const float* times, const int64_t* off
   }
   if (2 * cap >= (int64_t)0xFFFFFFFFll)
     return set_error(VGICP_ERR_INVALID_ARG, "more than 2^31-1 table slots");
+  // one buffer; its front is filled by the host in one copy: offsets, tables, and the
+  // zeroed counters
   size_t off = 0;
   auto take = [&](size_t bytes) {
     const size_t o = off;
     off = (off + std::max<size_t>(bytes, 1) + 255) & ~size_t(255);
     return o;
   };
+  const int G = times && split > 0.0 ? 2 : 1;
+  const int64_t n_groups = cap * G, n_words = n / 32 + 1;
   const size_t o_off = take(sizeof(int64_t) * (n_clouds + 1));
   const size_t o_base = take(sizeof(int64_t) * n_clouds);
   const size_t o_mask = take(sizeof(uint32_t) * n_clouds);
+  const size_t o_cursor = take(sizeof(uint32_t));
   const size_t o_status = take(sizeof(int32_t));
-  const size_t o_nout = take(sizeof(uint32_t));
-  const size_t o_oo = take(sizeof(uint32_t) * (n_clouds + 1));
+  const size_t upload = off;
+  const size_t o_oo = take(sizeof(uint32_t) * (n_clouds + 2));
   const size_t o_slots = take(sizeof(DsSlot) * cap);
-  const size_t o_gfirst = take(sizeof(uint32_t) * 2 * cap);
-  const size_t o_gmap = take(sizeof(uint32_t) * 2 * cap);
+  const size_t o_groups = take(sizeof(DsGroup) * n_groups);
   const size_t o_ptslot = take(sizeof(uint32_t) * n);
   const size_t o_ptgroup = take(sizeof(uint32_t) * n);
-  const size_t o_flag = take(sizeof(uint32_t) * n);
-  const size_t o_prefix = take(sizeof(uint32_t) * n);
-  const size_t o_gcount = take(sizeof(uint32_t) * n);
-  const size_t o_goff = take(sizeof(uint32_t) * n);
   const size_t o_list = take(sizeof(uint32_t) * n);
-  const size_t o_scan = take(sizeof(uint32_t) * scan_tmp_elems(n));
+  const size_t o_bitmap = take(sizeof(uint32_t) * n_words);
+  const size_t o_wscan = take(sizeof(uint32_t) * n_words);
+  const size_t o_scan = take(sizeof(uint32_t) * scan_tmp_elems(n_words));
+  std::vector<char> host(upload, 0);
+  std::memcpy(host.data() + o_off, offsets, sizeof(int64_t) * (n_clouds + 1));
+  std::memcpy(host.data() + o_base, base.data(), sizeof(int64_t) * n_clouds);
+  std::memcpy(host.data() + o_mask, mask.data(), sizeof(uint32_t) * n_clouds);
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   char* d = nullptr;
   VGICP_CUDA_TRY(device_malloc(reinterpret_cast<void**>(&d), off, st, true));
@@ -304,61 +458,58 @@ int vgicp_downsample(const float* points, const float* times, const int64_t* off
   int64_t* d_base = reinterpret_cast<int64_t*>(d + o_base);
   int32_t* d_status = reinterpret_cast<int32_t*>(d + o_status);
   DsSlot* d_slots = reinterpret_cast<DsSlot*>(d + o_slots);
+  DsGroup* d_groups = reinterpret_cast<DsGroup*>(d + o_groups);
   int rc = VGICP_OK;
-  cudaError_t e = cudaMemcpyAsync(d_off, offsets, sizeof(int64_t) * (n_clouds + 1),
-                                  cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(d_base, base.data(), sizeof(int64_t) * n_clouds, cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(U(o_mask), mask.data(), sizeof(uint32_t) * n_clouds,
-                        cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(d_status, 0, sizeof(int32_t), st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(U(o_gcount), 0, sizeof(uint32_t) * n, st);
+  // (a copy from pageable memory returns once the source is staged)
+  cudaError_t e = cudaMemcpyAsync(d, host.data(), upload, cudaMemcpyHostToDevice, st);
   if (e != cudaSuccess) rc = check_cuda(e, "downsample setup");
   const float inv_r = (float)(1.0 / resolution);
-  const int g = grid_of(n), gc = grid_of(cap);
+  const int g = grid_of(n);
+  const bool fused = n_words <= kScanWords;
   if (rc == VGICP_OK) {
-    ds_init_kernel<<<gc, kThreads, 0, st>>>(d_slots, cap, U(o_gfirst));
+    ds_init_kernel<<<grid_of(n_groups), kThreads, 0, st>>>(reinterpret_cast<uint4*>(d_slots), cap,
+                                                          reinterpret_cast<uint4*>(d_groups),
+                                                          n_groups);
     ds_insert_kernel<<<g, kThreads, 0, st>>>(points, n, d_off, n_clouds, inv_r, resolution,
                                              d_base, U(o_mask), d_slots, U(o_ptslot), d_status);
-    ds_group_kernel<<<g, kThreads, 0, st>>>(n, times, split, d_slots, U(o_ptslot), U(o_gfirst),
+    ds_group_kernel<<<g, kThreads, 0, st>>>(n, times, split, G, d_slots, U(o_ptslot), d_groups,
                                             U(o_ptgroup));
-    ds_flags_kernel<<<g, kThreads, 0, st>>>(n, U(o_ptgroup), U(o_gfirst), U(o_flag));
+    const int n_mark = grid_of(n_words * 32);
+    const int n_place = grid_of((n_groups + kPlacePer - 1) / kPlacePer);
+    ds_mark_kernel<<<n_mark + n_place, kThreads, 0, st>>>(n, n_words, n_mark, U(o_ptgroup),
+                                                         d_groups, n_groups, U(o_bitmap),
+                                                         U(o_cursor));
     count_launches(4);
-    rc = launch_exclusive_scan(U(o_flag), U(o_prefix), n, nullptr, U(o_scan), U(o_nout), st);
+    if (fused) {
+      ds_scatter_kernel<<<g + 1, kThreads, 0, st>>>(n, U(o_ptgroup), d_groups, U(o_list), n_words,
+                                                   U(o_bitmap), U(o_wscan), n_clouds, d_off,
+                                                   d_status, U(o_oo));
+      count_launches(1);
+    } else {
+      ds_popc_kernel<<<grid_of(n_words), kThreads, 0, st>>>(n_words, U(o_bitmap), U(o_wscan));
+      rc = launch_exclusive_scan(U(o_wscan), U(o_wscan), n_words, nullptr, U(o_scan), nullptr, st);
+      ds_scatter_large_kernel<<<grid_of(std::max<int64_t>(n, n_clouds + 1)), kThreads, 0, st>>>(
+          n, U(o_ptgroup), d_groups, U(o_list), U(o_bitmap), U(o_wscan), n_clouds, d_off, d_status,
+          U(o_oo));
+      count_launches(2);
+    }
   }
   if (rc == VGICP_OK) {
-    ds_assign_kernel<<<g, kThreads, 0, st>>>(n, U(o_flag), U(o_prefix), U(o_ptgroup), U(o_gmap));
-    // pt_slot is free now: the output voxel of each point
-    ds_count_kernel<<<g, kThreads, 0, st>>>(n, U(o_ptgroup), U(o_gmap), U(o_gcount), U(o_ptslot));
-    count_launches(2);
-    rc = launch_exclusive_scan(U(o_gcount), U(o_goff), n, U(o_nout), U(o_scan), nullptr, st);
-  }
-  if (rc == VGICP_OK) {
-    e = cudaMemsetAsync(U(o_flag), 0, sizeof(uint32_t) * n, st);  // the fill counters
-    if (e != cudaSuccess) rc = check_cuda(e, "cudaMemsetAsync");
-  }
-  if (rc == VGICP_OK) {
-    ds_scatter_kernel<<<g, kThreads, 0, st>>>(n, U(o_ptslot), U(o_goff), U(o_flag), U(o_list));
-    ds_finalize_kernel<<<g, kThreads, 0, st>>>(n, U(o_nout), points, times, U(o_gcount),
-                                               U(o_goff), U(o_list), out_points, out_times,
+    ds_finalize_kernel<<<g, kThreads, 0, st>>>(n, U(o_bitmap), U(o_wscan), U(o_ptgroup), d_groups,
+                                               points, times, U(o_list), out_points, out_times,
                                                out_counts);
-    ds_offsets_kernel<<<(n_clouds + 1 + 127) / 128, 128, 0, st>>>(n_clouds, n, d_off, U(o_prefix),
-                                                                   U(o_nout), U(o_oo));
-    count_launches(3);
+    count_launches(1);
     e = cudaGetLastError();
     if (e != cudaSuccess) rc = check_cuda(e, "downsample kernels");
   }
-  std::vector<uint32_t> oo((size_t)n_clouds + 1, 0u);
-  int32_t status = 0;
+  std::vector<uint32_t> oo((size_t)n_clouds + 2, 0u);  // the offsets, then the status
   if (rc == VGICP_OK) {
     e = cudaMemcpyAsync(oo.data(), U(o_oo), sizeof(uint32_t) * oo.size(), cudaMemcpyDeviceToHost,
                         st);
-    if (e == cudaSuccess)
-      e = cudaMemcpyAsync(&status, d_status, sizeof(int32_t), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) rc = check_cuda(e, "downsample results");
   }
+  const int32_t status = (int32_t)oo[(size_t)n_clouds + 1];
   e = cudaFreeAsync(d, st);
   if (rc == VGICP_OK && e != cudaSuccess) rc = check_cuda(e, "cudaFreeAsync");
   if (rc == VGICP_OK && status == VGICP_ERR_KEY_RANGE)
