@@ -531,12 +531,19 @@ int vgicp_linearize(const vgicp_map* map, const float* src_points, const float* 
   const size_t part_bytes = sizeof(double) * kPartialStride * std::max<int32_t>(n_items, 1);
   VGICP_CUDA_TRY(device_malloc(reinterpret_cast<void**>(&scratch), part_bytes + 256, st, true));
   L.partials = reinterpret_cast<double*>(scratch);
-  L.status = reinterpret_cast<int32_t*>(scratch + part_bytes);
-  cudaError_t e = cudaMemsetAsync(L.status, 0, 2 * sizeof(int32_t), st);
-  rc = e == cudaSuccess ? VGICP_OK : check_cuda(e, "cudaMemsetAsync");
-  if (rc == VGICP_OK) rc = launch_linearize(L, st);
-  if (rc == VGICP_OK)
-    rc = launch_reduce(L.partials, nullptr, n_items, 1, L.status, out, inliers, st);
+  cudaError_t e = cudaSuccess;
+  if (factor_in_one_launch(L)) {
+    rc = launch_factor(L, out, inliers, st);
+  } else {
+    if (needs_status(L)) {
+      L.status = reinterpret_cast<int32_t*>(scratch + part_bytes);
+      e = cudaMemsetAsync(L.status, 0, 2 * sizeof(int32_t), st);
+      rc = e == cudaSuccess ? VGICP_OK : check_cuda(e, "cudaMemsetAsync");
+    }
+    if (rc == VGICP_OK) rc = launch_linearize(L, st);
+    if (rc == VGICP_OK)
+      rc = launch_reduce(L.partials, nullptr, n_items, 1, L.status, out, inliers, st);
+  }
   e = cudaFreeAsync(scratch, st);
   if (rc == VGICP_OK && e != cudaSuccess) rc = check_cuda(e, "cudaFreeAsync");
   return rc;
@@ -814,6 +821,7 @@ extern "C" int vgicp_linearize_noalloc(const vgicp_map* map, const float* src_po
   L.ev_start = opts ? static_cast<cudaEvent_t>(opts->kernel_start) : nullptr;
   L.ev_stop = opts ? static_cast<cudaEvent_t>(opts->kernel_stop) : nullptr;
   L.partials = scratch;
+  if (factor_in_one_launch(L)) return launch_factor(L, out, inliers, st);
   L.status = reinterpret_cast<int32_t*>(scratch + (size_t)kNoAllocMaxItems * kPartialStride);
   // the array keeps the previous call's contents: the status word must start at
   // zero; every partial the reduction reads is written by this call

@@ -136,6 +136,10 @@ struct LinLaunch {
                                // producer withholds (0 = none)
 };
 int launch_linearize(const LinLaunch& L, cudaStream_t st);
+bool needs_status(const LinLaunch& L);  // else L.status may be null
+// A small single factor, linearization and reduction in one launch.
+bool factor_in_one_launch(const LinLaunch& L);
+int launch_factor(const LinLaunch& L, double* out, int64_t* inliers, cudaStream_t st);
 
 // Arms the one-shot wait test of the next staged-kernel launch
 // (vgicp_test_expire_waits).
@@ -149,13 +153,14 @@ int default_variant();
 
 // Sum each pair's partials over its items [span[p].x, span[p].y) in order and
 // expand to the 43-double result; span == nullptr means one pair over all
-// n_items_single items.  A nonzero *status turns every output into NaN.
+// n_items_single items.  A nonzero *status (with bad != 0: one equal to
+// bad) turns every output into NaN; status may be null.
 // Gradient modes: jr (n_pairs x 36, device, or null) gives J_r^T g instead of g,
 // gscale (n_pairs, device, or null) scales the gradient.
 int launch_reduce(const double* partials, const int2* span, int32_t n_items_single,
                   int64_t n_pairs, const int32_t* status, double* out, int64_t* inliers,
                   cudaStream_t st, int32_t mode = 0, const double* jr = nullptr,
-                  const double* gscale = nullptr);
+                  const double* gscale = nullptr, int32_t bad = 0);
 
 int device_sm_count();
 

@@ -30,6 +30,7 @@ struct vgicp_plan {
   int32_t variant = 0, item = 0, grid = 0;  // current launch shape
   int64_t n_items = 0;
   int64_t items_cap = 0;
+  int32_t evaluations = 0;       // differentiable evaluations so far (numbers them)
   // device
   char* d_block = nullptr;
   PairDesc* d_pd = nullptr;
@@ -152,14 +153,22 @@ int upload_poses(vgicp_plan* P, int b, cudaStream_t st) {
 // Pose of every factor for a differentiable evaluation, in binary64 on the
 // device: T_p = T0_p Exp(xi_p) (xi = null: T0_p), written as the factor's
 // descriptor, and J_r(xi_p) when jr is given.  A base pose that is not a finite
-// rigid transform, or a non-finite increment, sets the status word (all
-// outputs of the evaluation become NaN) and uses the identity.
-__global__ void compose_kernel(const double* __restrict__ base, const double* __restrict__ xi,
+// rigid transform, or a non-finite increment, writes this evaluation's number to the
+// status word (all its outputs become NaN) and uses the identity.  Also zeroes the
+// work-item counter behind the status word for the launch that follows.
+// One warp per CTA, and the Jacobians in CTAs of their own (blockIdx.y = 1): a
+// binary64 instruction occupies an SM's one unit for 16 cycles per warp, so four warps
+// on an SM, each doing both, took 44 us for a forward and a backward pass of 256
+// factors; now 32 us, the latency of one warp's chain (two sines and cosines, a
+// square root, divisions).
+constexpr int kComposeThreads = 32;
+__global__ void __launch_bounds__(kComposeThreads) compose_kernel(const double* __restrict__ base, const double* __restrict__ xi,
                                const int2* __restrict__ ms, int64_t n_pairs,
                                PairDesc* __restrict__ pd, double* __restrict__ jr,
-                               int32_t* __restrict__ status) {
+                               int32_t* __restrict__ status, int32_t number) {
   const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (p >= n_pairs) return;
+  if (p == 0 && blockIdx.y == 0) status[1] = 0;
   double T0[16], x[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0}, E[16], T[16];
   for (int i = 0; i < 16; ++i) T0[i] = base[16 * p + i];
   bool ok = se3::rigid(T0);
@@ -169,14 +178,17 @@ __global__ void compose_kernel(const double* __restrict__ base, const double* __
       ok = ok && isfinite(x[i]);
     }
   if (!ok) {
-    atomicExch(status, 2);
+    atomicExch(status, number);
     for (int i = 0; i < 16; ++i) T0[i] = (i % 5 == 0) ? 1.0 : 0.0;
     for (int i = 0; i < 6; ++i) x[i] = 0.0;
+  }
+  if (blockIdx.y == 1) {
+    se3::right_jacobian(x, jr + 36 * p);
+    return;
   }
   se3::expmap(x, E);
   se3::pose_mul(T0, E, T);
   pd[p] = se3::pair_desc(T, ms[p].x, ms[p].y);
-  if (jr) se3::right_jacobian(x, jr + 36 * p);
 }
 
 void drop_graph(vgicp_plan* P) {
@@ -337,6 +349,7 @@ int vgicp_plan_create(vgicp_map* const* maps, int32_t n_maps, const vgicp_cloud*
       (e = cudaEventCreateWithFlags(&P->uploaded[0], cudaEventDisableTiming)) != cudaSuccess ||
       (e = cudaEventCreateWithFlags(&P->uploaded[1], cudaEventDisableTiming)) != cudaSuccess ||
       (e = cudaStreamCreateWithFlags(&P->cap, cudaStreamNonBlocking)) != cudaSuccess ||
+      (e = cudaMemset(P->d_status, 0, 2 * sizeof(int32_t))) != cudaSuccess ||
       (e = cudaMemcpy(P->d_ms, ms.data(), sizeof(int2) * ms.size(),
                       cudaMemcpyHostToDevice)) != cudaSuccess ||
       (e = cudaMemcpy(P->d_md, P->md.data(), sizeof(MapDesc) * P->md.size(),
@@ -445,11 +458,12 @@ int vgicp_plan_evaluate(vgicp_plan* P, const double* base_poses, const double* x
   if (!P || !base_poses || !out) return set_error(VGICP_ERR_INVALID_ARG, "null plan, poses or out");
   if (mode < 1 || mode > 3) return set_error(VGICP_ERR_INVALID_ARG, "mode must be 1, 2 or 3");
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  VGICP_CUDA_TRY(cudaMemsetAsync(P->d_status, 0, 2 * sizeof(int32_t), st));
+  const int32_t number = P->evaluations = P->evaluations % INT32_MAX + 1;  // never 0
   double* jr = mode >= 2 && xi ? P->d_jr : nullptr;
   const int64_t n = P->n_pairs;
-  compose_kernel<<<(unsigned)((n + 127) / 128), 128, 0, st>>>(base_poses, xi, P->d_ms, n, P->d_pd,
-                                                              jr, P->d_status);
+  const dim3 grid((unsigned)((n + kComposeThreads - 1) / kComposeThreads), jr ? 2 : 1);
+  compose_kernel<<<grid, kComposeThreads, 0, st>>>(base_poses, xi, P->d_ms, n, P->d_pd, jr,
+                                                  P->d_status, number);
   VGICP_CUDA_TRY(cudaGetLastError());
   count_launches(1);
   LinLaunch L = launch_of(P);
@@ -458,7 +472,7 @@ int vgicp_plan_evaluate(vgicp_plan* P, const double* base_poses, const double* x
   if (rc) return rc;
   // the caller's inlier buffer, or the plan's own
   return launch_reduce(P->d_partials, P->d_span, 0, n, P->d_status, out,
-                       inliers ? inliers : P->d_inl, st, mode, jr, grad_scale);
+                       inliers ? inliers : P->d_inl, st, mode, jr, grad_scale, number);
 }
 
 int vgicp_plan_info(const vgicp_plan* P, int32_t* variant, int32_t* item_points, int32_t* grid,

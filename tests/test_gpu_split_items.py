@@ -53,3 +53,21 @@ def test_points_without_a_voxel_and_not_finite(dev):  # noqa: F811
     ra, rb = a.execute(poses), b.execute(poses)
     assert bool(torch.isfinite(ra.out).all())
     assert torch.equal(ra.out, rb.out) and torch.equal(ra.inliers, rb.inliers)
+
+
+@pytest.mark.parametrize("n,tile", [(0, 0), (1, 0), (31, 0), (255, 0), (256, 0), (257, 0), (2048, 0),
+                                    (8191, 0), (8192, 0), (8193, 0), (16384, 0), (16385, 0),
+                                    (16385, 512), (32768, 512), (32769, 512), (700, 100)])
+def test_single_factor_in_one_launch(dev, n, tile):  # noqa: F811
+    """A small single factor is one cluster's work; a grid request keeps the general
+    launches.  Same sums, with the scratch of vgicp_linearize and without allocation."""
+    w = synth.with_surface_covariances(
+        synth.outdoor_submaps(seed=8, n_submaps=2, n_min=33000, n_max=33000, neighbours=1))
+    (tp, tc), (sp, sc) = w.clouds.cloud(int(w.pairs[0, 0])), w.clouds.cloud(int(w.pairs[0, 1]))
+    vm = api.VoxelMap.build(cu(tp), cu(tc), 1.0)
+    src = (cu(sp[:n]), cu(sc[:n]))
+    a = api.linearize(vm, *src, w.poses[0], tile=tile)
+    b = api.linearize(vm, *src, w.poses[0], tile=tile, grid=456)
+    assert torch.equal(a.out, b.out) and torch.equal(a.inliers, b.inliers)
+    if n > 100:
+        assert int(a.inliers) > 0
