@@ -1111,6 +1111,7 @@ int size_lookup_tables(MapSet* s, cudaStream_t st) {
                                  cudaMemcpyDeviceToHost, st));
   VGICP_CUDA_TRY(cudaStreamSynchronize(st));
   s->vslot_base.assign((size_t)s->n_maps + 1, 0);
+  s->vox.assign((size_t)s->n_maps, 0u);
   int64_t total = 0;
   for (int32_t m = 0; m < s->n_maps; ++m) {
     const uint64_t V = vb[m + 1] >= vb[m] ? vb[m + 1] - vb[m] : 0;
@@ -1121,6 +1122,7 @@ int size_lookup_tables(MapSet* s, cudaStream_t st) {
     uint64_t c = 16;
     while (c < kLookupLoad * V || c < 2 * nm) c <<= 1;
     s->vslot_base[m] = total;
+    s->vox[m] = (uint32_t)V;
     total += (int64_t)c;
   }
   s->vslot_base[s->n_maps] = total;

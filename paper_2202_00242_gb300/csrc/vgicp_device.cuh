@@ -134,6 +134,40 @@ __device__ __forceinline__ uint32_t hash_key(int kx, int ky, int kz) {
   return h ^ (h >> 16);
 }
 
+// Occupancy block of 4 x 4 x 4 voxels (27-neighbour linearization): bit z * 16 + y * 4
+// + x of `bits` for the voxel at (x, y, z) of the block; its record is `first` plus the
+// number of lower bits set.  key = 0: empty.
+struct __align__(32) BlockSlot {
+  unsigned long long key;
+  unsigned long long bits;
+  uint32_t first;
+  uint32_t pad[3];
+};
+constexpr int kBlockProbes = 256;  // a block lies within this many slots of its home
+// Block coordinates are voxel keys >> 2, one further out on either side allowed.
+constexpr int kBlockBias = (kKeyBias >> 2) + 1;
+__device__ __forceinline__ unsigned long long block_key(int bx, int by, int bz) {
+  return (1ull << 63) | ((unsigned long long)(uint32_t)(bx + kBlockBias) << 40) |
+         ((unsigned long long)(uint32_t)(by + kBlockBias) << 20) |
+         (unsigned long long)(uint32_t)(bz + kBlockBias);
+}
+
+// A target map's blocks and what they are built from (all device pointers).
+struct BlockMap {
+  const unsigned long long* vkeys;  // keys by voxel id
+  const uint32_t* vbase;            // this map's first voxel id, and the next map's
+  const uint32_t* lslot_of;         // lookup slot by voxel id (into vslots)
+  const VSlot* vslots;
+  BlockSlot* table;                 // mask + 1 slots, zeroed
+  float4* recs;                     // rec_cap x 3: (mu', -), (l00, l10, l20, l11), (l21, l22, -, -)
+  uint32_t* block_of;               // rec_cap: block slot by voxel
+  uint32_t* state;                  // zeroed: [0] nonzero: does not fit; [1] records placed;
+                                    // [2] blocks
+  uint32_t* any;                    // zeroed: nonzero if some map of the call does not fit
+  uint32_t mask;
+  uint32_t rec_cap;
+};
+
 // Clamp a float to the int range before conversion, so out-of-range values map
 // to out-of-range keys instead of wrapping.
 __device__ __forceinline__ int clamp_to_int(float f) {

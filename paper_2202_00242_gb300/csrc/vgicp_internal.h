@@ -46,6 +46,7 @@ struct MapSet {
   std::vector<uint32_t> cap;       // n_maps
   std::vector<int64_t> vslot_base; // n_maps + 1: lookup-table regions, sized from the voxel
   int64_t vcap_total = 0;          //   counts of the first build (empty before it)
+  std::vector<uint32_t> vox;       // n_maps: voxels of the first build
   // device: per-map metadata
   int64_t* d_point_off = nullptr;  // n_maps + 1
   int64_t* d_slot_base = nullptr;  // n_maps
@@ -108,6 +109,11 @@ int launch_exclusive_scan(const uint32_t* in, uint32_t* out, int64_t n_max,
                           cudaStream_t st);
 size_t scan_tmp_elems(int64_t n_max);
 
+// ---- kernels (vgicp_blocks.cu) ---------------------------------------------
+// Blocks a table should have room for, given a map's voxels; the table build.
+uint32_t block_capacity(int64_t voxels);
+int launch_blocks(const BlockMap* d_maps, int32_t n_maps, int64_t max_voxels, cudaStream_t st);
+
 // ---- kernels (vgicp_linearize.cu) ----------------------------------------
 struct LinLaunch {
   const WorkItem* items;     // null: uniform items of pair 0 (single factor)
@@ -116,6 +122,9 @@ struct LinLaunch {
   const PairDesc* pairs;     // null: use `single`
   const MapDesc* maps;       // null: use `single_map`
   const SrcDesc* srcs;       // null: use `single_src`
+  const BlockMap* blocks;    // 27 neighbours: the maps' occupancy blocks, or null
+  const uint32_t* blocks_any;  // with blocks: nonzero if some map has none (status then
+                               //   holds a second work-item counter, [2])
   PairDesc single;
   MapDesc single_map;
   SrcDesc single_src;

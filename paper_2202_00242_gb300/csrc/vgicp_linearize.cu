@@ -799,10 +799,14 @@ __global__ void __launch_bounds__(kSimpleThreads, simple_ctas(NEIGH, MODE))
   __shared__ int next_item;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint64_t pol = policy_evict_last_l();
+  // with occupancy blocks only the items of the maps that have none are left
+  if (NEIGH == 27 && L.blocks && *L.blocks_any == 0u) return;
 
   for (int it = blockIdx.x; it < L.n_items;) {
     int pair, begin, end;
     tma::item_bounds(L, it, pair, begin, end);
+    const bool skip = NEIGH == 27 && L.blocks && L.blocks[L.pairs[pair].map].state[0] == 0u;
+    if (skip) end = begin;
     if (threadIdx.x == 0) {
       const PairDesc* pd = L.pairs ? L.pairs + pair : &L.single;
       const MapDesc md = L.maps ? L.maps[pd->map] : L.single_map;
@@ -981,7 +985,7 @@ __global__ void __launch_bounds__(kSimpleThreads, simple_ctas(NEIGH, MODE))
     if (threadIdx.x == 0)
       next_item = L.status ? (int)gridDim.x + atomicAdd(L.status + 1, 1) : L.n_items;
     __syncthreads();
-    if (threadIdx.x < kAcc) {
+    if (threadIdx.x < kAcc && !skip) {
       double s = 0.0;
       for (int w = 0; w < kSimpleThreads / 32; ++w) s += (double)red[w][threadIdx.x];
       L.partials[(int64_t)it * kPartialStride + threadIdx.x] = s;
@@ -990,6 +994,205 @@ __global__ void __launch_bounds__(kSimpleThreads, simple_ctas(NEIGH, MODE))
     __syncthreads();
   }
 }
+
+// ---------------------------------------------------------------------------
+// 27 neighbours from occupancy blocks (vgicp_blocks.cu): one point per thread, work
+// items claimed as in the per-point kernel.  The masks of the 1 - 8 blocks around a
+// point are shifted so that bit z * 16 + y * 4 + x says whether neighbour (x, y, z) of
+// the 3 x 3 x 3 block exists, and its set bits in ascending order are the neighbours in
+// the order of the per-point kernel (dz, dy, dx), so the sums are the same bit for bit.
+// A neighbour's record is found from its block's mask and first record, which wait in
+// shared memory; the next neighbour's record is loaded while the current one's term is
+// evaluated.
+// Bounded by issue, with 20 of 32 lanes active (a lane has 0 to 27 terms): 96M source
+// points of 48 large-map submaps 13.1 -> 9.4 ms, and 0.2 ms to build the blocks; of
+// the 9.4 ms the search takes 2.3 (the probes took 8.4), the records' places 1.3, their
+// loads 1.2, the terms 4.6.  Four or two CTAs per SM: 10.2, 10.7 ms.
+// ---------------------------------------------------------------------------
+namespace blocks {
+// Moves the cells that a block holds of a window of three, starting at cell `lo` (0..3)
+// of the first block, to their place in the window, along the axis whose cells are W
+// bits apart (all_lowest: the lowest cell of the axis everywhere): second = false: cells
+// lo .. 3 down by lo, true: cells 0 .. lo - 2 up by 4 - lo.
+template <int W>
+__device__ __forceinline__ uint64_t to_window(uint64_t m, int lo, bool second) {
+  // the first three cells of every group of four, along this axis
+  constexpr uint64_t kCell = W == 1 ? 0x1111111111111111ull : W == 4 ? 0x000F000F000F000Full
+                                                                     : 0x000000000000FFFFull;
+  constexpr uint64_t kThree = kCell | (kCell << W) | (kCell << (2 * W));
+  if (second) {  // cells 0 .. lo - 2 (lo >= 2)
+    const uint64_t keep = lo == 3 ? kCell | (kCell << W) : kCell;
+    return (m & keep) << (W * (4 - lo));
+  }
+  const uint64_t keep = lo == 0 ? kThree : lo == 1 ? kThree << W : lo == 2 ? (kCell | (kCell << W)) << (2 * W)
+                                                                          : kCell << (3 * W);
+  return (m & keep) >> (W * lo);
+}
+
+constexpr int kCtas = 3;  // per SM
+template <int MODE>
+__global__ void __launch_bounds__(kSimpleThreads, kCtas)
+    linearize_blocks_kernel(const __grid_constant__ LinLaunch L) {
+  __shared__ float red[kSimpleThreads / 32][kAcc];
+  // each thread's half blocks (4 x 4 x 2), hz * 4 + cy * 2 + cx: mask, first record
+  __shared__ uint2 s_half[12][kSimpleThreads];
+  __shared__ ItemConst ic;
+  __shared__ BlockMap bm;
+  __shared__ int next_item;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint64_t pol = policy_evict_last_l();
+
+  for (int it = blockIdx.x; it < L.n_items;) {
+    int pair, begin, end;
+    tma::item_bounds(L, it, pair, begin, end);
+    const PairDesc* pd = L.pairs + pair;
+    const bool skip = L.blocks[pd->map].state[0] != 0u;  // the same for the CTA
+    if (threadIdx.x == 0) {
+      const MapDesc md = L.maps[pd->map];
+      const SrcDesc sd = L.srcs[pd->src];
+#pragma unroll
+      for (int k = 0; k < 9; ++k) ic.R[k] = pd->R[k];
+      ic.t[0] = pd->t[0];
+      ic.t[1] = pd->t[1];
+      ic.t[2] = pd->t[2];
+      ic.tmax = pd->tmax;
+      ic.inv_r = md.inv_r;
+      ic.margin_scale = md.margin_scale;
+      ic.pts = sd.pts;
+      ic.covs = sd.covs;
+      ic.pd = pd;
+      ic.r = md.r;
+      bm = L.blocks[pd->map];
+    }
+    __syncthreads();
+    float acc[kAcc];
+#pragma unroll
+    for (int k = 0; k < kAcc; ++k) acc[k] = 0.0f;
+    Pose32 P;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) P.R[k] = uniform(ic.R[k]);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) P.t[k] = uniform(ic.t[k]);
+    P.tmax = uniform(ic.tmax);
+    MapDesc md;
+    md.inv_r = uniform(ic.inv_r);
+    md.margin_scale = uniform(ic.margin_scale);
+    const BlockSlot* const table = uniform(bm.table);
+    const float4* const recs = uniform(bm.recs);
+    const uint32_t mask = uniform(bm.mask);
+
+    for (int64_t p = skip ? end : begin + (int)threadIdx.x; p < end; p += kSimpleThreads) {
+      const float* pt = ic.pts + 3 * p;
+      const float x = __ldg(pt + 0), y = __ldg(pt + 1), z = __ldg(pt + 2);
+      const float2* cv = reinterpret_cast<const float2*>(ic.covs + 6 * p);
+      const float2 c01 = __ldg(cv + 0), c23 = __ldg(cv + 1), c45 = __ldg(cv + 2);
+      const float c[6] = {c01.x, c01.y, c23.x, c23.y, c45.x, c45.y};
+      const float qx = fmaf(P.R[0], x, fmaf(P.R[1], y, fmaf(P.R[2], z, P.t[0])));
+      const float qy = fmaf(P.R[3], x, fmaf(P.R[4], y, fmaf(P.R[5], z, P.t[1])));
+      const float qz = fmaf(P.R[6], x, fmaf(P.R[7], y, fmaf(P.R[8], z, P.t[2])));
+      int kx, ky, kz;
+      source_key(P, ic.pd, md_of_item(md, ic.r), x, y, z, qx, qy, qz, kx, ky, kz);
+      // no neighbour is in the key range beyond one voxel outside it
+      if (kx < kKeyMin - 1 || kx > kKeyMax + 1 || ky < kKeyMin - 1 || ky > kKeyMax + 1 ||
+          kz < kKeyMin - 1 || kz > kKeyMax + 1)
+        continue;
+      const int lx = (kx - 1) & 3, ly = (ky - 1) & 3, lz = (kz - 1) & 3;
+      const int bx = (kx - 1) >> 2, by = (ky - 1) >> 2, bz = (kz - 1) >> 2;
+      uint64_t occ = 0ull;  // window bits
+#pragma unroll 1
+      for (int cz = 0; cz <= (lz >= 2); ++cz) {
+        uint64_t slab = 0ull;
+#pragma unroll 1
+        for (int cy = 0; cy <= (ly >= 2); ++cy) {
+          uint64_t rows = 0ull;
+          // the two blocks of a row: their home slots loaded together
+          uint32_t a[2][8];
+          uint32_t h[2];
+#pragma unroll
+          for (int cx = 0; cx < 2; ++cx) {
+            h[cx] = hash_key(bx + cx, by + cy, bz + cz) & mask;
+            if (cx == 0 || lx >= 2) ld_v8(table + h[cx], pol, a[cx]);
+          }
+#pragma unroll
+          for (int cx = 0; cx < 2; ++cx) {
+            if (cx == 1 && lx < 2) continue;
+            const unsigned long long key = block_key(bx + cx, by + cy, bz + cz);
+            unsigned long long k = slot_key(a[cx]);
+            for (int q = 1; q < kBlockProbes && k != key && k != 0ull; ++q) {
+              h[cx] = (h[cx] + 1) & mask;
+              ld_v8(table + h[cx], pol, a[cx]);
+              k = slot_key(a[cx]);
+            }
+            if (k != key) continue;
+            const uint64_t bits = (uint64_t)a[cx][2] | ((uint64_t)a[cx][3] << 32);
+            // the window reaches half blocks 0 - 2 in z (cells lz .. lz + 2 <= 5)
+            const int b = cz * 8 + cy * 2 + cx;
+            s_half[b][threadIdx.x] = make_uint2(a[cx][2], a[cx][4]);
+            if (cz == 0)
+              s_half[b + 4][threadIdx.x] =
+                  make_uint2(a[cx][3], a[cx][4] + (uint32_t)__popc(a[cx][2]));
+            rows |= to_window<1>(bits, lx, cx == 1);
+          }
+          slab |= to_window<4>(rows, ly, cy == 1);
+        }
+        occ |= to_window<16>(slab, lz, cz == 1);
+      }
+      if (occ == 0ull) continue;
+      // the neighbours, two slabs of the window (32 bits) and then the third
+      uint32_t now = (uint32_t)occ, then = (uint32_t)(occ >> 32);
+      int z0 = lz;
+      auto next = [&]() {  // record of the lowest bit, which is cleared
+        if (now == 0u) {
+          now = then;
+          then = 0u;
+          z0 = lz + 2;
+        }
+        const int wbit = __ffs((int)now) - 1;
+        now &= now - 1u;
+        const int wx = lx + (wbit & 3), wy = ly + ((wbit >> 2) & 3), wz = z0 + (wbit >> 4);
+        const int bit = (wz & 1) * 16 + (wy & 3) * 4 + (wx & 3);
+        const uint2 m = s_half[(wz >> 1) * 4 + (wy >> 2) * 2 + (wx >> 2)][threadIdx.x];
+        return recs + 3 * (m.y + (uint32_t)__popc(m.x & ((1u << bit) - 1u)));
+      };
+      const float4* rec = next();
+      float4 n0 = __ldg(rec), n1 = __ldg(rec + 1), n2 = __ldg(rec + 2);
+      while (true) {
+        const float4 r0 = n0, r1 = n1, r2 = n2;
+        const bool more = (now | then) != 0u;
+        if (more) {
+          rec = next();
+          n0 = __ldg(rec);
+          n1 = __ldg(rec + 1);
+          n2 = __ldg(rec + 2);
+        }
+        term<MODE>(acc, P, x, y, z, c, qx, qy, qz, r0, r1, r2);
+        if (!more) break;
+      }
+    }
+
+#pragma unroll
+    for (int k = 0; k < kAcc; ++k) {
+      float v = acc[k];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
+      acc[k] = v;
+    }
+    if (lane == 0) {
+#pragma unroll
+      for (int k = 0; k < kAcc; ++k) red[warp][k] = acc[k];
+    }
+    if (threadIdx.x == 0) next_item = (int)gridDim.x + atomicAdd(L.status + 1, 1);
+    __syncthreads();
+    if (threadIdx.x < kAcc && !skip) {
+      double s = 0.0;
+      for (int w = 0; w < kSimpleThreads / 32; ++w) s += (double)red[w][threadIdx.x];
+      L.partials[(int64_t)it * kPartialStride + threadIdx.x] = s;
+    }
+    it = next_item;  // read between the two barriers; rewritten only after the second
+    __syncthreads();
+  }
+}
+}  // namespace blocks
 
 template <int NEIGH, int MODE>
 void launch_simple(const LinLaunch& L, int grid, cudaStream_t st) {
@@ -1721,6 +1924,17 @@ int launch_linearize(const LinLaunch& L, cudaStream_t st) {
   int grid = L.grid > 0 ? L.grid : linearize_grid(L.neighbours, variant, L.mode);
   grid = std::min(grid, L.n_items);
   if (L.ev_start) VGICP_CUDA_TRY(cudaEventRecord(L.ev_start, st));
+  LinLaunch Lb = L;
+  if (L.neighbours == 27 && L.blocks) {
+    // the maps with occupancy blocks, then (below) the items of those without
+    const int bgrid = L.grid > 0 ? grid : std::min(device_sm_count() * blocks::kCtas, L.n_items);
+    if (L.mode == 0) blocks::linearize_blocks_kernel<0><<<bgrid, kSimpleThreads, 0, st>>>(L);
+    else if (L.mode == 1) blocks::linearize_blocks_kernel<1><<<bgrid, kSimpleThreads, 0, st>>>(L);
+    else if (L.mode == 2) blocks::linearize_blocks_kernel<2><<<bgrid, kSimpleThreads, 0, st>>>(L);
+    else blocks::linearize_blocks_kernel<3><<<bgrid, kSimpleThreads, 0, st>>>(L);
+    count_launches(1);
+    Lb.status = L.status + 1;  // the second work-item counter
+  }
   if (split_items(L, variant)) {
     const unsigned ctas = (unsigned)L.n_items * split::kCtas;
     if (L.mode == 0) split::linearize_split_kernel<0><<<ctas, split::kThreads, 0, st>>>(L);
@@ -1730,9 +1944,9 @@ int launch_linearize(const LinLaunch& L, cudaStream_t st) {
   } else if (L.mode != 0) {
     // cost / gradient evaluations use the per-point kernel
     if (L.neighbours == 27) {
-      if (L.mode == 1) launch_simple<27, 1>(L, grid, st);
-      else if (L.mode == 2) launch_simple<27, 2>(L, grid, st);
-      else launch_simple<27, 3>(L, grid, st);
+      if (L.mode == 1) launch_simple<27, 1>(Lb, grid, st);
+      else if (L.mode == 2) launch_simple<27, 2>(Lb, grid, st);
+      else launch_simple<27, 3>(Lb, grid, st);
     } else {
       if (L.mode == 1) launch_simple<1, 1>(L, grid, st);
       else if (L.mode == 2) launch_simple<1, 2>(L, grid, st);
@@ -1740,7 +1954,7 @@ int launch_linearize(const LinLaunch& L, cudaStream_t st) {
       else launch_simple<1, 4>(L, grid, st);
     }
   } else if (L.neighbours == 27) {
-    launch_simple<27, 0>(L, grid, st);
+    launch_simple<27, 0>(Lb, grid, st);
   } else if (variant == 1) {
     launch_simple<1, 0>(L, grid, st);
   } else if (variant == 3 && !L.corr_out && !L.qkey_out) {
