@@ -119,7 +119,6 @@ int create_set(const int64_t* offsets, int32_t n_maps, double resolution,
   const size_t o_vkeys = take(sizeof(unsigned long long) * n);
   const size_t o_status = take(sizeof(int32_t));
   const size_t o_num_vox = take(sizeof(uint32_t));
-  const size_t o_num_valid = take(sizeof(uint32_t));
   const size_t o_pt_slot = take(sizeof(uint32_t) * n);
   const size_t o_flag = take(sizeof(uint32_t) * n);
   const size_t o_vcount = take(sizeof(uint32_t) * n);
@@ -159,7 +158,6 @@ int create_set(const int64_t* offsets, int32_t n_maps, double resolution,
   s->d_vkeys = reinterpret_cast<unsigned long long*>(b + o_vkeys);
   s->d_status = reinterpret_cast<int32_t*>(b + o_status);
   s->d_num_voxels = reinterpret_cast<uint32_t*>(b + o_num_vox);
-  s->d_num_valid = reinterpret_cast<uint32_t*>(b + o_num_valid);
   s->d_pt_slot = reinterpret_cast<uint32_t*>(b + o_pt_slot);
   s->d_flag = reinterpret_cast<uint32_t*>(b + o_flag);
   s->d_vcount = reinterpret_cast<uint32_t*>(b + o_vcount);

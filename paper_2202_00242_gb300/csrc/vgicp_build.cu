@@ -14,11 +14,11 @@
 //             (a scan of the words' popcounts), so voxels are numbered in order
 //             of first appearance, map by map; each first point gives its voxel
 //             its count, key and, in the slot, its id
-//   sort      per map chunk: the voxels in Morton order of their keys (rank)
-//   scan      offsets of the voxels' point lists, in rank order and by voxel
+//             (and per map: lookup-table capacity from the voxel count)
+//   sort      per map chunk: the voxels in Morton order of their keys (rank), and
+//             the offsets of their point lists, in rank order and by voxel
 //   scatter   per point: append its index to its voxel's list; the voxel's
 //             last point empties its build-table slot
-//   capacity  per map: lookup-table capacity from the voxel count
 //   finalize  per voxel, in rank order: sort its list, sum means and
 //             covariances (exactly, else in binary64 in ascending point index),
 //             divide by N, round to float32; copy the points into the voxel-
@@ -70,7 +70,8 @@ __device__ __forceinline__ void set_status(int32_t* status, int32_t code) {
   atomicCAS(status, 0, code);
 }
 
-__global__ void init_slots_kernel(Slot* __restrict__ slots, int64_t cap_total) {
+__global__ void init_slots_kernel(Slot* __restrict__ slots, int64_t cap_total, int32_t* status) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) *status = 0;
   for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < cap_total;
        s += (int64_t)gridDim.x * blockDim.x) {
     Slot e;
@@ -130,7 +131,9 @@ __global__ void insert_kernel(const float* __restrict__ pts, int64_t n_total,
 // set only on claimed slots), which leaves the tables empty.  (The build table
 // is emptied by the scatter of every build.)
 __global__ void reset_tables_kernel(int64_t n_max, const uint32_t* __restrict__ n_vox,
-                                    const uint32_t* __restrict__ lslot_of, VSlot* vslots) {
+                                    const uint32_t* __restrict__ lslot_of, VSlot* vslots,
+                                    int32_t* status) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) *status = 0;
   const int64_t V = *n_vox;
   for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < V && v < n_max;
        v += (int64_t)gridDim.x * blockDim.x) {
@@ -206,12 +209,6 @@ __device__ __forceinline__ void insert_lookup(uint32_t v, unsigned long long key
     set_status(status, VGICP_ERR_HASH_FULL);
     return;
   }
-  VSlot& sl = t[h];
-  sl.vid = v;
-  sl.count = c;
-  sl.mu[0] = q[0];
-  sl.mu[1] = q[1];
-  sl.mu[2] = q[2];
   // the Cholesky factor L of C' (the linearization forms R^T C' R as (R^T L)(R^T L)^T);
   // a non-positive pivot (a semi-definite C') leaves its column zero
   const float l00 = q[3] > 0.f ? sqrtf(q[3]) : 0.f;
@@ -222,12 +219,13 @@ __device__ __forceinline__ void insert_lookup(uint32_t v, unsigned long long key
   const float l21 = l11 > 0.f ? (q[7] - l20 * l10) / l11 : 0.f;
   const float p22 = q[8] - l20 * l20 - l21 * l21;
   const float l22 = p22 > 0.f ? sqrtf(p22) : 0.f;
-  sl.cov[0] = l00;
-  sl.cov[1] = l10;
-  sl.cov[2] = l20;
-  sl.cov[3] = l11;
-  sl.cov[4] = l21;
-  sl.cov[5] = l22;
+  // whole words of the slot (key and spill aside): as scalar stores the slot took
+  // finalize of the global map from 1.09 to 1.15 ms
+  char* sl = reinterpret_cast<char*>(t + h);
+  reinterpret_cast<VSlot*>(sl)->mu[0] = q[0];
+  *reinterpret_cast<float4*>(sl + 16) = make_float4(q[1], q[2], l00, l10);
+  *reinterpret_cast<float4*>(sl + 32) = make_float4(l20, l11, l21, l22);
+  *reinterpret_cast<uint4*>(sl + 48) = make_uint4(v, c, 0u, 0u);
 }
 
 // Per-voxel sums and the grouped cloud.  A CTA takes 128 consecutive ranks,
@@ -347,9 +345,9 @@ __device__ __forceinline__ void write_record(uint32_t v, uint32_t o, uint32_t c,
 }
 
 __global__ void __launch_bounds__(kFinThreads) finalize_kernel(
-    int64_t n_max, const uint32_t* __restrict__ n_vox, const uint32_t* __restrict__ n_valid,
-    const float* __restrict__ pts, const float* __restrict__ covs,
-    const uint32_t* __restrict__ vorder, const uint32_t* __restrict__ goff,
+    int64_t n_max, const uint32_t* __restrict__ n_vox, const float* __restrict__ pts,
+    const float* __restrict__ covs, const uint32_t* __restrict__ vorder,
+    const uint32_t* __restrict__ goff,
     uint32_t* __restrict__ plist, float4* __restrict__ recs, float* gpts, float* gcovs,
     const unsigned long long* __restrict__ vkeys, int32_t n_maps,
     const uint32_t* __restrict__ vbase, const int64_t* __restrict__ slot_base,
@@ -358,7 +356,7 @@ __global__ void __launch_bounds__(kFinThreads) finalize_kernel(
   __shared__ uint32_t stage[kFinStage];
   __shared__ int seg_map[2];
   const int64_t V = min((int64_t)*n_vox, n_max);
-  const uint32_t total = *n_valid;  // end of the last list (goff[V] is not stored)
+  const uint32_t total = (uint32_t)n_max;  // end of the last list (goff[V] is not stored)
   for (int64_t r0 = (int64_t)blockIdx.x * kFinThreads; r0 < V; r0 += (int64_t)gridDim.x * kFinThreads) {
     const int64_t r1 = min(V, r0 + kFinThreads);
     // list bounds from consecutive offsets: no dependent load through vorder
@@ -387,7 +385,9 @@ __global__ void __launch_bounds__(kFinThreads) finalize_kernel(
     // 2. gather into the grouped cloud
     const uint32_t* lst = staged ? stage : plist + seg0;
     for (uint32_t i = threadIdx.x; i < len; i += kFinThreads) {
-      const int64_t j = lst[i];
+      // (a point without a voxel, which the build reports, leaves a gap behind its map's
+      // last list, whatever it holds)
+      const int64_t j = min(lst[i], total - 1u);
       const float x = __ldg(pts + 3 * j), y = __ldg(pts + 3 * j + 1), z = __ldg(pts + 3 * j + 2);
       const float2* cv = reinterpret_cast<const float2*>(covs + 6 * j);
       const float2 c0 = __ldg(cv), c1 = __ldg(cv + 1), c2 = __ldg(cv + 2);
@@ -453,9 +453,9 @@ __device__ __forceinline__ void add_lane(float* hi, float* lo, bool& exact, int 
 // sets of short lists.
 constexpr uint32_t kFinSerial = 64;
 __global__ void __launch_bounds__(kFinThreads) finalize_long_kernel(
-    int64_t n_max, const uint32_t* __restrict__ n_vox, const uint32_t* __restrict__ n_valid,
-    const float* __restrict__ pts, const float* __restrict__ covs,
-    const uint32_t* __restrict__ vorder, const uint32_t* __restrict__ goff,
+    int64_t n_max, const uint32_t* __restrict__ n_vox, const float* __restrict__ pts,
+    const float* __restrict__ covs, const uint32_t* __restrict__ vorder,
+    const uint32_t* __restrict__ goff,
     uint32_t* __restrict__ plist, float4* __restrict__ recs, float* gpts, float* gcovs,
     const unsigned long long* __restrict__ vkeys, int32_t n_maps,
     const uint32_t* __restrict__ vbase, const int64_t* __restrict__ slot_base,
@@ -464,8 +464,8 @@ __global__ void __launch_bounds__(kFinThreads) finalize_long_kernel(
   __shared__ uint32_t stage[kFinStage];
   __shared__ uint32_t list_at[kFinThreads];  // first entry of each list, in the segment
   const int64_t V = min((int64_t)*n_vox, n_max);
-  const uint32_t total = *n_valid;  // end of the last list (goff[V] is not stored)
-  const uint32_t avg = (uint32_t)((int64_t)total / max((int64_t)1, V));
+  const uint32_t total = (uint32_t)n_max;  // end of the last list (goff[V] is not stored)
+  const uint32_t avg = (uint32_t)(n_max / max((int64_t)1, V));
   int R = kFinThreads;
   while (R > 4 && (uint32_t)R * avg > 512u) R >>= 1;
   const int per = kFinThreads / R;  // threads per voxel (1 .. 32)
@@ -490,7 +490,7 @@ __global__ void __launch_bounds__(kFinThreads) finalize_long_kernel(
     __syncthreads();
     for (uint32_t i = threadIdx.x; i < len; i += kFinThreads) {
       const uint32_t id = staged ? stage[i] : plist[seg0 + i];
-      const int64_t j = id;
+      const int64_t j = min(id, total - 1u);  // (see above)
       const float x = __ldg(pts + 3 * j), y = __ldg(pts + 3 * j + 1), z = __ldg(pts + 3 * j + 2);
       const float2* cv = reinterpret_cast<const float2*>(covs + 6 * j);
       const float2 c0 = __ldg(cv), c1 = __ldg(cv + 1), c2 = __ldg(cv + 2);
@@ -561,8 +561,10 @@ __device__ __forceinline__ uint32_t spread10(uint32_t x) {
   return x;
 }
 // One CTA (of 1024 threads) or one cluster of 8 CTAs (of 256) per (map, chunk): the
-// chunk's voxels sorted by Morton code (ties by voxel id); vorder[rank] = v and
-// gcount[rank] = the voxel's point count.
+// chunk's voxels sorted by Morton code (ties by voxel id); vorder[rank] = v, goff[rank] =
+// the offset of its point list (the map's first point plus the counts of the ranks
+// before; the lists of a map fill its range of points), also stored by voxel for the
+// scatter, as (offset << 32 | fill 0).
 //
 // A stable radix sort, least significant digit first, the elements spread evenly
 // over the CTAs' shared memory.  A warp holds 32 J consecutive elements, J per lane
@@ -627,7 +629,8 @@ template <int CTAS, int THREADS>
 __global__ void __launch_bounds__(THREADS) morton_sort_kernel(
     const int2* __restrict__ chunks, const uint32_t* __restrict__ vbase,
     const unsigned long long* __restrict__ vkeys, const uint32_t* __restrict__ vcount,
-    uint32_t* __restrict__ vorder, uint32_t* __restrict__ gcount) {
+    const int64_t* __restrict__ point_off, uint32_t* __restrict__ vorder,
+    uint32_t* __restrict__ goff, unsigned long long* __restrict__ bfill) {
   constexpr int kWarps = THREADS / 32, kGroups = THREADS / kDigits, kEach = kWarps / kGroups;
   constexpr int kItems = kMortonChunk / (CTAS * THREADS);
   static_assert(kEach == 8 && kItems % 2 == 0, "scan and register layout");
@@ -814,16 +817,67 @@ __global__ void __launch_bounds__(THREADS) morton_sort_kernel(
     if (ctas > 1u) cluster_sync();
     else __syncthreads();
   }
-  for (uint32_t i = threadIdx.x; i < mine; i += THREADS) {
-    const uint32_t v = first + (uint32_t)S.idx[i];
-    vorder[first + c0 + i] = v;
-    gcount[first + c0 + i] = vcount[v];
+  // points of the map's earlier chunks
+  uint32_t base = 0u;
+  for (uint32_t i = threadIdx.x; i < lo; i += THREADS) base += vcount[v0 + i];
+  base = __reduce_add_sync(0xFFFFFFFFu, base);
+  if (lane == 0) S.warp[w] = base;
+  __syncthreads();
+  base = (uint32_t)point_off[m];
+  for (int i = 0; i < kWarps; ++i) base += S.warp[i];
+  // list offsets: a scan of the counts in rank order, 32 ranks of the warp's at a time,
+  // then over the warps and the CTAs before
+  uint32_t off[kItems], run = 0u;
+#pragma unroll
+  for (int j = 0; j < kItems; ++j) {
+    off[j] = 0u;
+    if (j < (int)J) {  // the same for all lanes
+      const uint32_t e = e0 + 32u * j;
+      uint32_t n = 0u;
+      if (e < mine) {
+        const uint32_t v = first + (uint32_t)S.idx[e];
+        vorder[first + c0 + e] = v;
+        n = vcount[v];
+      }
+      uint32_t inc = n;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, inc, o);
+        if (lane >= o) inc += y;
+      }
+      off[j] = run + inc - n;
+      run += __shfl_sync(0xFFFFFFFFu, inc, 31);
+    }
+  }
+  __syncthreads();  // S.warp has been read
+  if (lane == 0) S.warp[w] = run;
+  __syncthreads();
+  uint32_t all = 0u;
+  for (int i = 0; i < kWarps; ++i) {
+    if (i < w) base += S.warp[i];
+    all += S.warp[i];
+  }
+  if (ctas > 1u) {
+    if (threadIdx.x < ctas) st_cluster(smem_of_rank(&S.bits[rank], threadIdx.x), all);
+    cluster_sync();
+#pragma unroll
+    for (int i = 0; i < CTAS; ++i)
+      if (i < (int)rank) base += S.bits[i];
+  }
+#pragma unroll
+  for (int j = 0; j < kItems; ++j) {
+    const uint32_t e = e0 + 32u * j;
+    if (j < (int)J && e < mine) {
+      const uint32_t o = base + off[j];
+      goff[first + c0 + e] = o;
+      bfill[first + (uint32_t)S.idx[e]] = (unsigned long long)o << 32;
+    }
   }
 }
 
 // Launches the sort with CTAS CTAs of THREADS threads per chunk.
 template <int CTAS, int THREADS>
-int launch_sort(const MapSet* s, uint32_t* vorder, uint32_t* gcount, cudaStream_t st) {
+int launch_sort(const MapSet* s, uint32_t* vorder, unsigned long long* bfill, cudaStream_t st) {
   constexpr int kBytes = (int)sizeof(SortSmem<CTAS, THREADS>);
   auto* kernel = morton_sort_kernel<CTAS, THREADS>;
   if (kBytes > 48 * 1024) {  // above the default limit: opt in once per device
@@ -852,7 +906,8 @@ int launch_sort(const MapSet* s, uint32_t* vorder, uint32_t* gcount, cudaStream_
   cfg.numAttrs = CTAS > 1 ? 1 : 0;
   VGICP_CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel, (const int2*)s->d_chunks, (const uint32_t*)s->d_vbase,
                                     (const unsigned long long*)s->d_vkeys,
-                                    (const uint32_t*)s->d_vcount, vorder, gcount));
+                                    (const uint32_t*)s->d_vcount, (const int64_t*)s->d_point_off,
+                                    vorder, s->d_goff, bfill));
   return VGICP_OK;
 }
 
@@ -862,17 +917,22 @@ __device__ __forceinline__ uint32_t lookup_capacity(uint32_t nvox) {
   return c;
 }
 
-// Per map (blockIdx.y): lookup-table capacity from its voxel count; with
-// clear_all, every slot of the map's region emptied (the first build, whose
-// region is fresh; later builds find the region empty after the reset).
+// Slots a build uses of a map's region, which the first build sized; a rebuild with
+// more voxels runs at a higher load factor (an insertion past max_probe reports
+// VGICP_ERR_HASH_FULL).
+__device__ __forceinline__ uint32_t table_capacity(uint32_t nvox, uint32_t region) {
+  return min(lookup_capacity(nvox), region);
+}
+
+// First build (and empty sets), per map (blockIdx.y): lookup-table capacity from its
+// voxel count; with clear_all, every slot of the map's region emptied (fresh memory;
+// later builds find the region empty after the reset).
 __global__ void vslot_init_kernel(const int64_t* __restrict__ slot_base,
                                   const uint32_t* __restrict__ vbase, VSlot* vslots,
                                   uint32_t* __restrict__ vmask, int32_t clear_all) {
   const int m = blockIdx.y;
-  // the region was sized by the first build; a rebuild with more voxels runs at a
-  // higher load factor (an insertion past max_probe reports VGICP_ERR_HASH_FULL)
   const uint32_t region = (uint32_t)(slot_base[m + 1] - slot_base[m]);
-  const uint32_t cap = min(lookup_capacity(vbase[m + 1] - vbase[m]), region);
+  const uint32_t cap = table_capacity(vbase[m + 1] - vbase[m], region);
   if (clear_all) {
     VSlot* t = vslots + slot_base[m];
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < region;
@@ -978,34 +1038,6 @@ __global__ void scan_tiles_kernel(const uint32_t* in, uint32_t* out, int64_t n_m
   }
 }
 
-// Last pass of the scan of the rank-ordered counts: goff[r] = the offset of rank
-// r's list, also stored by voxel for the scatter, as (base << 32 | fill 0).
-__global__ void scan_lists_kernel(const uint32_t* __restrict__ gcount, uint32_t* __restrict__ goff,
-                                  int64_t n_max, const uint32_t* __restrict__ n_dev,
-                                  const uint32_t* __restrict__ sums,
-                                  const uint32_t* __restrict__ vorder,
-                                  unsigned long long* __restrict__ bfill) {
-  const int64_t n = scan_len(n_max, n_dev);
-  const int64_t b0 = (int64_t)blockIdx.x * kScanTile + threadIdx.x * kScanPerThread;
-  uint32_t v[kScanPerThread];
-  uint32_t s = 0;
-#pragma unroll
-  for (int k = 0; k < kScanPerThread; ++k) {
-    v[k] = (b0 + k < n) ? gcount[b0 + k] : 0u;
-    s += v[k];
-  }
-  __shared__ uint32_t total;
-  uint32_t run = block_exclusive<kScanThreads>(s, &total) + sums[blockIdx.x];
-#pragma unroll
-  for (int k = 0; k < kScanPerThread; ++k) {
-    if (b0 + k < n) {
-      goff[b0 + k] = run;
-      bfill[vorder[b0 + k]] = (unsigned long long)run << 32;  // fill 0
-    }
-    run += v[k];
-  }
-}
-
 // ---- first-appearance numbering -----------------------------------------
 // A point is its voxel's first if its index is the smallest of the voxel (the
 // build-table slot holds that index after the insert).  The first points are
@@ -1013,8 +1045,8 @@ __global__ void scan_lists_kernel(const uint32_t* __restrict__ gcount, uint32_t*
 // of marked points before its first point (an exclusive scan of the words'
 // popcounts), so voxels are numbered in order of first appearance, map by map.
 
-// One thread per point; every warp is whole (the grid covers n rounded up to
-// 32), so the ballot sees all 32 lanes.
+// One thread per point; every warp is whole, so the ballot sees all 32 lanes.  The
+// grid covers the word of index n, which the ranks below read.
 __global__ void first_bits_kernel(const uint32_t* __restrict__ pt_slot,
                                   const Slot* __restrict__ slots, int64_t n,
                                   uint32_t* __restrict__ bitmap) {
@@ -1025,7 +1057,7 @@ __global__ void first_bits_kernel(const uint32_t* __restrict__ pt_slot,
     f = ps != kNoSlot && slots[ps].vid == (uint32_t)i;
   }
   const unsigned b = __ballot_sync(0xFFFFFFFFu, f);
-  if ((threadIdx.x & 31) == 0 && i < n) bitmap[i >> 5] = b;
+  if ((threadIdx.x & 31) == 0 && (i >> 5) <= (n >> 5)) bitmap[i >> 5] = b;
 }
 
 __global__ void popc_words_kernel(const uint32_t* __restrict__ bitmap, int64_t n_words,
@@ -1061,17 +1093,67 @@ __global__ void assign_ids_kernel(const uint32_t* __restrict__ bitmap,
   }
 }
 
-// vbase[m] = voxels of the maps before m; vbase[n_maps] and *n_vox = all.
+// vbase[m] = voxels of the maps before m; vbase[n_maps] and *n_vox = all.  With vmask
+// (a rebuild) also each map's lookup-table mask.
+__device__ __forceinline__ void map_ranges(int m, int32_t n_maps, int64_t n_total,
+                                           const int64_t* __restrict__ point_off,
+                                           const uint32_t* bitmap, const uint32_t* wscan,
+                                           uint32_t* __restrict__ vbase,
+                                           uint32_t* __restrict__ n_vox,
+                                           const int64_t* __restrict__ vslot_base,
+                                           uint32_t* __restrict__ vmask) {
+  const uint32_t v =
+      first_rank(bitmap, wscan, (uint32_t)(m < n_maps ? point_off[m] : n_total));
+  vbase[m] = v;
+  if (m == n_maps) {
+    *n_vox = v;
+  } else if (vmask) {
+    const uint32_t next =
+        first_rank(bitmap, wscan, (uint32_t)(m + 1 < n_maps ? point_off[m + 1] : n_total));
+    vmask[m] = table_capacity(next - v, (uint32_t)(vslot_base[m + 1] - vslot_base[m])) - 1u;
+  }
+}
 __global__ void vbase_kernel(int32_t n_maps, int64_t n_total, const int64_t* __restrict__ point_off,
                              const uint32_t* __restrict__ bitmap,
                              const uint32_t* __restrict__ wscan, uint32_t* __restrict__ vbase,
-                             uint32_t* __restrict__ n_vox) {
+                             uint32_t* __restrict__ n_vox, const int64_t* __restrict__ vslot_base,
+                             uint32_t* __restrict__ vmask) {
   const int m = blockIdx.x * blockDim.x + threadIdx.x;
-  if (m > n_maps) return;
-  const int64_t o = m < n_maps ? point_off[m] : n_total;
-  const uint32_t v = first_rank(bitmap, wscan, (uint32_t)o);
-  vbase[m] = v;
-  if (m == n_maps) *n_vox = v;
+  if (m <= n_maps)
+    map_ranges(m, n_maps, n_total, point_off, bitmap, wscan, vbase, n_vox, vslot_base, vmask);
+}
+
+// The words' popcounts scanned and the maps' ranges, by one CTA: five launches in one
+// while the words are few (200,000 points: 2 us; kNumberWords take 6 us, the scan's
+// launches for as many 9).
+constexpr int64_t kNumberWords = 32768;
+constexpr int kNumberThreads = 1024, kNumberPer = 8;
+__global__ void __launch_bounds__(kNumberThreads) number_kernel(
+    const uint32_t* bitmap, int64_t n_words, uint32_t* wscan, int32_t n_maps, int64_t n_total,
+    const int64_t* __restrict__ point_off, uint32_t* __restrict__ vbase,
+    uint32_t* __restrict__ n_vox, const int64_t* __restrict__ vslot_base,
+    uint32_t* __restrict__ vmask) {
+  __shared__ uint32_t total;
+  uint32_t carry = 0u;
+  for (int64_t w0 = 0; w0 < n_words; w0 += kNumberThreads * kNumberPer) {
+    const int64_t a = w0 + (int64_t)threadIdx.x * kNumberPer;
+    uint32_t c[kNumberPer], sum = 0u;
+#pragma unroll
+    for (int k = 0; k < kNumberPer; ++k) {
+      c[k] = a + k < n_words ? (uint32_t)__popc(bitmap[a + k]) : 0u;
+      sum += c[k];
+    }
+    uint32_t run = carry + block_exclusive<kNumberThreads>(sum, &total);
+#pragma unroll
+    for (int k = 0; k < kNumberPer; ++k) {
+      if (a + k < n_words) wscan[a + k] = run;
+      run += c[k];
+    }
+    carry += total;
+    __syncthreads();  // the CTA's words are visible to it; `total` may be rewritten
+  }
+  for (int m = threadIdx.x; m <= n_maps; m += kNumberThreads)
+    map_ranges(m, n_maps, n_total, point_off, bitmap, wscan, vbase, n_vox, vslot_base, vmask);
 }
 
 // One thread per element (no grid-stride cap): CTAs are dispatched roughly in
@@ -1155,14 +1237,12 @@ int launch_build(MapSet* s, const float* points, const float* covs, cudaStream_t
   if (was_built) {
     // empty the slots of the previous build's voxels
     reset_tables_kernel<<<gv, kThreads, 0, st>>>(n, s->d_num_voxels, s->d_lslot_of,
-                                                 s->d_vslots);
-    count_launches(1);
-  } else if (s->cap_total > 0) {
-    init_slots_kernel<<<grid_for(s->cap_total, kThreads), kThreads, 0, st>>>(s->d_slots,
-                                                                          s->cap_total);
-    count_launches(1);
+                                                 s->d_vslots, s->d_status);
+  } else {
+    init_slots_kernel<<<grid_for(s->cap_total, kThreads), kThreads, 0, st>>>(
+        s->d_slots, s->cap_total, s->d_status);
   }
-  VGICP_CUDA_TRY(cudaMemsetAsync(s->d_status, 0, sizeof(int32_t), st));
+  count_launches(1);
   if (n == 0) {
     VGICP_CUDA_TRY(cudaMemsetAsync(s->d_num_voxels, 0, sizeof(uint32_t), st));
     VGICP_CUDA_TRY(cudaMemsetAsync(s->d_vbase, 0, sizeof(uint32_t) * (s->n_maps + 1), st));
@@ -1190,19 +1270,26 @@ int launch_build(MapSet* s, const float* points, const float* covs, cudaStream_t
     const int64_t n_words = n / 32 + 1;
     uint32_t* bitmap = s->d_flag;
     uint32_t* wscan = s->d_vfill;
-    VGICP_CUDA_TRY(cudaMemsetAsync(bitmap + n / 32, 0, sizeof(uint32_t), st));
-    first_bits_kernel<<<grid_for(n, kThreads), kThreads, 0, st>>>(s->d_pt_slot, s->d_slots, n,
-                                                                  bitmap);
-    popc_words_kernel<<<grid_for(n_words, kThreads), kThreads, 0, st>>>(bitmap, n_words, wscan);
-    rc = launch_exclusive_scan(wscan, wscan, n_words, nullptr, s->d_scan_tmp, nullptr, st);
-    if (rc != VGICP_OK) return rc;
+    uint32_t* vmask = was_built ? s->d_vmask : nullptr;  // the first build sizes the tables below
+    first_bits_kernel<<<grid_for(32 * n_words, kThreads), kThreads, 0, st>>>(s->d_pt_slot,
+                                                                           s->d_slots, n, bitmap);
+    if (n_words <= kNumberWords) {
+      number_kernel<<<1, kNumberThreads, 0, st>>>(bitmap, n_words, wscan, s->n_maps, n,
+                                                  s->d_point_off, s->d_vbase, s->d_num_voxels,
+                                                  s->d_vslot_base, vmask);
+    } else {
+      popc_words_kernel<<<grid_for(n_words, kThreads), kThreads, 0, st>>>(bitmap, n_words, wscan);
+      rc = launch_exclusive_scan(wscan, wscan, n_words, nullptr, s->d_scan_tmp, nullptr, st);
+      if (rc != VGICP_OK) return rc;
+      vbase_kernel<<<(s->n_maps + 1 + 127) / 128, 128, 0, st>>>(
+          s->n_maps, n, s->d_point_off, bitmap, wscan, s->d_vbase, s->d_num_voxels,
+          s->d_vslot_base, vmask);
+      count_launches(1);
+    }
     assign_ids_kernel<<<g, kThreads, 0, st>>>(bitmap, wscan, n, s->d_pt_slot, s->d_slots,
                                               s->d_vcount, s->d_vkeys);
-    vbase_kernel<<<(s->n_maps + 1 + 127) / 128, 128, 0, st>>>(s->n_maps, n, s->d_point_off,
-                                                              bitmap, wscan, s->d_vbase,
-                                                              s->d_num_voxels);
     VGICP_CUDA_TRY(cudaGetLastError());
-    count_launches(4);
+    count_launches(3);
   }
   if (!s->d_vblock) {
     rc = size_lookup_tables(s, st);
@@ -1212,51 +1299,36 @@ int launch_build(MapSet* s, const float* points, const float* covs, cudaStream_t
   // the lists, then the per-voxel sums (which also write the grouped clouds).
   // d_vfill (the numbering's word scan) is dead after the id assignment.
   uint32_t* vorder = s->d_voff;
-  uint32_t* gcount = s->d_vfill;
   // the lists' (base << 32 | fill) words, by voxel: in the record storage, which
   // finalize fills only after the scatter (8 of its 48 B per voxel)
   unsigned long long* bfill = reinterpret_cast<unsigned long long*>(s->d_recs);
   // a cluster per chunk while that leaves two SMs or more to a chunk (figures at the
   // kernel)
-  rc = 2 * s->n_chunks <= device_sm_count() ? launch_sort<8, 256>(s, vorder, gcount, st)
-                                            : launch_sort<1, 1024>(s, vorder, gcount, st);
+  rc = 2 * s->n_chunks <= device_sm_count() ? launch_sort<8, 256>(s, vorder, bfill, st)
+                                            : launch_sort<1, 1024>(s, vorder, bfill, st);
   if (rc != VGICP_OK) return rc;
   VGICP_CUDA_TRY(cudaGetLastError());
-  // list offsets in rank order, and by voxel
-  {
-    const int64_t nb = (n + kScanTile - 1) / kScanTile;
-    scan_tile_sums_kernel<<<(unsigned)nb, kScanThreads, 0, st>>>(gcount, n, s->d_num_voxels,
-                                                                 s->d_scan_tmp);
-    scan_sums_kernel<<<1, kScanSumsThreads, 0, st>>>(s->d_scan_tmp, nb, s->d_num_valid);
-    scan_lists_kernel<<<(unsigned)nb, kScanThreads, 0, st>>>(gcount, s->d_goff, n,
-                                                             s->d_num_voxels, s->d_scan_tmp,
-                                                             vorder, bfill);
-    VGICP_CUDA_TRY(cudaGetLastError());
-    count_launches(3);
-  }
   scatter_kernel<<<g, kThreads, 0, st>>>(n, s->d_pt_slot, s->d_slots, bfill, s->d_plist);
-  int64_t max_cap = 16;
-  for (int32_t m = 0; m < s->n_maps; ++m)
-    max_cap = std::max<int64_t>(max_cap, s->vslot_base[m + 1] - s->vslot_base[m]);
-  // the first build empties the whole lookup region; later ones set the masks only
-  const unsigned gx =
-      was_built ? 1u : (unsigned)std::min<int64_t>(64, (max_cap + kThreads - 1) / kThreads);
-  vslot_init_kernel<<<dim3(gx, s->n_maps), kThreads, 0, st>>>(s->d_vslot_base, s->d_vbase,
-                                                             s->d_vslots, s->d_vmask,
-                                                             was_built ? 0 : 1);
+  if (!was_built) {  // empty the whole lookup region and set the masks
+    int64_t max_cap = 16;
+    for (int32_t m = 0; m < s->n_maps; ++m)
+      max_cap = std::max<int64_t>(max_cap, s->vslot_base[m + 1] - s->vslot_base[m]);
+    const unsigned gx = (unsigned)std::min<int64_t>(64, (max_cap + kThreads - 1) / kThreads);
+    vslot_init_kernel<<<dim3(gx, s->n_maps), kThreads, 0, st>>>(s->d_vslot_base, s->d_vbase,
+                                                               s->d_vslots, s->d_vmask, 1);
+    count_launches(1);
+  }
   // sums, records, grouped clouds and the lookup tables
   // large sets of short lists (the first build's average) keep the kernel that sorts
   // them a thread per voxel (figures at finalize_long_kernel)
   const auto finalize =
       s->avg_list > 10 || n < 500000 ? finalize_long_kernel : finalize_kernel;
   finalize<<<g, kFinThreads, 0, st>>>(
-      n, s->d_num_voxels, s->d_num_valid, points, covs, vorder, s->d_goff, s->d_plist, s->d_recs,
+      n, s->d_num_voxels, points, covs, vorder, s->d_goff, s->d_plist, s->d_recs,
       s->d_gpts, s->d_gcovs, s->d_vkeys, s->n_maps, s->d_vbase, s->d_vslot_base, s->d_vmask,
       s->max_probe, s->d_vslots, s->d_lslot_of, s->d_status);
   VGICP_CUDA_TRY(cudaGetLastError());
-  // insert, sort, scatter, vslot init, finalize (+ reset or init: 1; numbering: 4;
-  // the two scans: 3 each)
-  count_launches(5);
+  count_launches(4);  // insert, sort, scatter, finalize
   s->built = true;
   return VGICP_OK;
 }

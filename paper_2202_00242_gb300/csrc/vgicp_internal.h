@@ -81,7 +81,6 @@ struct MapSet {
   int32_t n_chunks = 0;
   uint32_t* d_scan_tmp = nullptr; // scan block sums
   uint32_t* d_num_voxels = nullptr;  // 1 (total V)
-  uint32_t* d_num_valid = nullptr;   // 1 (points placed in a voxel)
   size_t scan_tmp_elems = 0;
   void* d_block = nullptr;        // single allocation holding everything above but d_vslots
   void* d_vblock = nullptr;       // the lookup tables (allocated by the first build)

@@ -132,6 +132,19 @@ __global__ void copy_words_kernel(uint4* __restrict__ dst, const uint4* __restri
     dst[i] = src[i];
 }
 
+// The plan's results to the caller's buffers (either may be null).
+__global__ void copy_results_kernel(double* __restrict__ out, int64_t* __restrict__ inliers,
+                                    const double* __restrict__ src_out,
+                                    const int64_t* __restrict__ src_inl, int64_t n_out,
+                                    int64_t n_pairs) {
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (i < n_out) {
+    if (out) out[i] = src_out[i];
+  } else if (i < n_out + n_pairs) {
+    if (inliers) inliers[i - n_out] = src_inl[i - n_out];
+  }
+}
+
 // The poses go to the device through a kernel that reads the pinned staging
 // buffer, not through a copy engine: a host-to-device copy queued there would
 // wait behind whatever large upload the caller has in flight (for instance the
@@ -443,12 +456,13 @@ int vgicp_plan_execute(vgicp_plan* P, const double* poses, double* out, int64_t*
   VGICP_CUDA_TRY(cudaGraphLaunch(P->exec, st));
   count_launches(2);  // linearize + reduce
   if (kernel_stop) VGICP_CUDA_TRY(cudaEventRecord(static_cast<cudaEvent_t>(kernel_stop), st));
-  if (out)
-    VGICP_CUDA_TRY(cudaMemcpyAsync(out, P->d_out, sizeof(double) * 43 * P->n_pairs,
-                                   cudaMemcpyDeviceToDevice, st));
-  if (inliers)
-    VGICP_CUDA_TRY(cudaMemcpyAsync(inliers, P->d_inl, sizeof(int64_t) * P->n_pairs,
-                                   cudaMemcpyDeviceToDevice, st));
+  if (out || inliers) {
+    const int64_t n_out = 43 * (int64_t)P->n_pairs, n = n_out + P->n_pairs;
+    copy_results_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(out, inliers, P->d_out,
+                                                                    P->d_inl, n_out, P->n_pairs);
+    VGICP_CUDA_TRY(cudaGetLastError());
+    count_launches(1);
+  }
   return VGICP_OK;
 }
 
