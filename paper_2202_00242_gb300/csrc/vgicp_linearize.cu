@@ -27,14 +27,18 @@
 // (ragged tails of the clouds, pairs with few inliers) do not leave CTAs idle.
 //
 // Kernels (the autotuner picks among the 1-neighbour ones per factor set):
-//   1  per-point: one point per thread, item constants in shared memory so that
-//      3 CTAs of 256 threads fit per SM; the default and usually the fastest;
+//   1  per-point: one point per thread, item constants in uniform registers so that
+//      4 CTAs of 256 threads fit per SM; the default and usually the fastest;
 //   2  staged: a producer warp streams tiles of points and covariances into
 //      shared memory with bulk asynchronous copies (cp.async.bulk + mbarrier);
 //      consumer warps look up, compact the hits and evaluate from shared memory;
 //   3  compacting: the per-point lookup, with the hits queued per warp in shared
 //      memory and evaluated 32 at a time (no idle lanes on misses);
-//   27 neighbours: the per-point kernel with the 27 lookups in a loop.
+//   27 neighbours: the per-point kernel with the 27 lookups in a loop, or, for large
+//      batches, the neighbours taken from occupancy blocks (namespace blocks).
+// Chosen by size, with the same results bit for bit:
+//   few items: a cluster of 8 CTAs per item (namespace split);
+//   a small single factor: items and their sum in one launch (namespace factor).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -1688,6 +1692,150 @@ __global__ void __cluster_dims__(kCtas, 1, 1) __launch_bounds__(kThreads, 2)
 }
 }  // namespace split
 
+// ---------------------------------------------------------------------------
+// Work items for at most two CTAs per SM (one neighbour): a CTA per item, four points
+// per thread at a time (two with two CTAs per SM) with their lookups in flight
+// together, and the next ones loaded while these are evaluated.
+//
+// The per-point kernel hides its loads behind other warps.  With one or two CTAs per SM
+// there are too few, and a thread's 64 points of a 16K item, each waiting for its
+// stream and then for its lookup, set the time.  At two CTAs per SM a thread may have
+// 128 registers, at one 255: room for the lookups of two or four points and for the next
+// points.  Each thread keeps its points and adds their terms in their order, so the
+// sums are those of the per-point kernel bit for bit.  Bounded by the latency of a
+// round (a lookup, the terms).  A plan's execution, factors of 16,000 points, maps as
+// sources / unsorted clouds: 152 factors 102 / 104 -> 63 / 66 us, 300 factors
+// 113 / 129 -> 86 / 98 us.
+// ---------------------------------------------------------------------------
+namespace ahead {
+// kPer: points per thread and round
+template <int MODE, int kPer>
+__global__ void __launch_bounds__(kSimpleThreads, 4 / kPer)
+    linearize_ahead_kernel(const __grid_constant__ LinLaunch L) {
+  __shared__ float red[kSimpleThreads / 32][kAcc];
+  __shared__ ItemConst ic;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int it = blockIdx.x;
+  const uint64_t pol = policy_evict_last_l();
+  int pair, begin, end;
+  tma::item_bounds(L, it, pair, begin, end);
+  if (threadIdx.x == 0) {
+    const PairDesc* pd = L.pairs ? L.pairs + pair : &L.single;
+    const MapDesc md = L.maps ? L.maps[pd->map] : L.single_map;
+    const SrcDesc sd = L.srcs ? L.srcs[pd->src] : L.single_src;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) ic.R[k] = pd->R[k];
+    ic.t[0] = pd->t[0];
+    ic.t[1] = pd->t[1];
+    ic.t[2] = pd->t[2];
+    ic.tmax = pd->tmax;
+    ic.inv_r = md.inv_r;
+    ic.margin_scale = md.margin_scale;
+    ic.mask = *md.vmask;
+    ic.vslots = md.vslots;
+    ic.pts = sd.pts;
+    ic.covs = sd.covs;
+    ic.pd = pd;
+    ic.r = md.r;
+    ic.max_probe = md.max_probe;
+  }
+  __syncthreads();
+  Pose32 P;
+#pragma unroll
+  for (int k = 0; k < 9; ++k) P.R[k] = uniform(ic.R[k]);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) P.t[k] = uniform(ic.t[k]);
+  P.tmax = uniform(ic.tmax);
+  MapDesc md;
+  md.inv_r = uniform(ic.inv_r);
+  md.margin_scale = uniform(ic.margin_scale);
+  md.vslots = uniform(ic.vslots);
+  const uint32_t mask = uniform(ic.mask);
+  const float* const pts = uniform(ic.pts + 3 * (int64_t)begin);
+  const float* const covs = uniform(ic.covs + 6 * (int64_t)begin);
+  const int64_t n = end - begin;
+
+  float acc[kAcc];
+#pragma unroll
+  for (int k = 0; k < kAcc; ++k) acc[k] = 0.0f;
+
+  float next[kPer][9];  // the points of the round to come: mean, covariance
+  auto load = [&](int64_t i0) {
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) {
+      const int64_t i = i0 + u * kSimpleThreads;
+      if (i < n) {
+        const float* pt = pts + 3 * i;
+        const float2* cv = reinterpret_cast<const float2*>(covs + 6 * i);
+        next[u][0] = __ldg(pt + 0);
+        next[u][1] = __ldg(pt + 1);
+        next[u][2] = __ldg(pt + 2);
+        const float2 c01 = __ldg(cv + 0), c23 = __ldg(cv + 1), c45 = __ldg(cv + 2);
+        next[u][3] = c01.x; next[u][4] = c01.y; next[u][5] = c23.x;
+        next[u][6] = c23.y; next[u][7] = c45.x; next[u][8] = c45.y;
+      }
+    }
+  };
+  load(threadIdx.x);
+  for (int64_t i0 = threadIdx.x; i0 < n; i0 += kPer * kSimpleThreads) {
+    float s[kPer][9], q[kPer][3];
+    uint32_t h[kPer], a[kPer][8], b[kPer][4];
+    unsigned long long key[kPer];
+    bool live[kPer];
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) {
+#pragma unroll
+      for (int k = 0; k < 9; ++k) s[u][k] = next[u][k];
+      live[u] = i0 + u * kSimpleThreads < n;
+      if (!live[u]) continue;
+      const float x = s[u][0], y = s[u][1], z = s[u][2];
+      q[u][0] = fmaf(P.R[0], x, fmaf(P.R[1], y, fmaf(P.R[2], z, P.t[0])));
+      q[u][1] = fmaf(P.R[3], x, fmaf(P.R[4], y, fmaf(P.R[5], z, P.t[1])));
+      q[u][2] = fmaf(P.R[6], x, fmaf(P.R[7], y, fmaf(P.R[8], z, P.t[2])));
+      int kx, ky, kz;
+      source_key(P, ic.pd, md_of_item(md, ic.r), x, y, z, q[u][0], q[u][1], q[u][2], kx, ky, kz);
+      live[u] = key_in_range(kx) && key_in_range(ky) && key_in_range(kz);
+      if (live[u]) {
+        key[u] = pack_key(kx, ky, kz);
+        h[u] = hash_key(kx, ky, kz) & mask;
+        ld_slot(md.vslots + h[u], pol, a[u], b[u]);
+      }
+    }
+    load(i0 + kPer * kSimpleThreads);
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) {
+      if (!live[u]) continue;
+      unsigned long long t = slot_key(a[u]);
+      for (int p = 1; t != key[u] && t != kEmptyKey && (p > 1 || a[u][kSlotSpill] != 0u) &&
+                      p < ic.max_probe;
+           ++p) {
+        h[u] = (h[u] + 1) & mask;
+        ld_slot(md.vslots + h[u], pol, a[u], b[u]);
+        t = slot_key(a[u]);
+      }
+      if (t != key[u]) continue;
+      float4 r0, r1, r2;
+      slot_gaussian(a[u], b[u], r0, r1, r2);
+      term<MODE>(acc, P, s[u][0], s[u][1], s[u][2], s[u] + 3, q[u][0], q[u][1], q[u][2], r0, r1, r2);
+    }
+  }
+
+#pragma unroll
+  for (int k = 0; k < kAcc; ++k) {
+    float v = acc[k];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
+    if (lane == 0) red[warp][k] = v;
+  }
+  __syncthreads();
+  if (threadIdx.x < kAcc) {
+    double v = 0.0;
+    for (int w = 0; w < kSimpleThreads / 32; ++w) v += (double)red[w][threadIdx.x];
+    L.partials[(int64_t)it * kPartialStride + threadIdx.x] = v;
+  }
+}
+}  // namespace ahead
+
 // Term `lane` (its sum s) of a linearization to its places in the 43-value result.
 __device__ __forceinline__ void write_result(int lane, double s, bool failed, double* o,
                                              int64_t* inliers) {
@@ -1884,13 +2032,31 @@ int linearize_grid(int neighbours, int variant, int mode) {
 
 // Whether a launch goes to the cluster-per-item kernel: the per-point kernel's
 // results (variant 1), at least four points per thread in a full item, and at most
-// three items to four SMs.  Linearization with the per-pair sums, cluster per item
-// against per-point (items of 16K, factors of 20,000 points; 152 SMs): 2 items 27
-// against 71 us, 20 items 28 / 75, 40 items 38 / 75, 76 items 50 / 75, 120 items
-// 68 / 75, 152 items 79 / 75.
+// three items to eight SMs, that is three of its CTAs to an SM.  A plan's execution,
+// factors of 16,000 points, cluster per item against the kernel of namespace ahead:
+// 40 items 48 / 51 us, 56 items 50 / 51, 76 items 71 / 53, 112 items 100 / 60.
 static bool split_items(const LinLaunch& L, int variant) {
   return L.neighbours != 27 && variant == 1 && L.mode <= 3 && L.grid <= 0 && !L.corr_out &&
-         !L.qkey_out && L.item_size >= 4 * kSimpleThreads && 4 * L.n_items <= 3 * device_sm_count();
+         !L.qkey_out && L.item_size >= 4 * kSimpleThreads && 8 * L.n_items <= 3 * device_sm_count();
+}
+
+// Points per thread of a launch that goes to the kernel of namespace ahead instead of the
+// per-point one, or 0: four where every item has an SM of its own, two up to two items
+// per SM.  Four against two points: 76 items 53 / 57 us, 152 items 63 / 70.  Above two items
+// per SM the items' waves count (350 items: 126 us by the per-point kernel, two waves here),
+// and for full grids the per-point kernel's 32 warps per SM hide more.
+static int ahead_items(const LinLaunch& L, int variant) {
+  if (L.neighbours == 27 || variant != 1 || L.mode > 3 || L.grid > 0 || L.corr_out || L.qkey_out ||
+      L.item_size < 4 * kSimpleThreads)
+    return 0;
+  return L.n_items <= device_sm_count() ? 4 : L.n_items <= 2 * device_sm_count() ? 2 : 0;
+}
+
+template <int MODE>
+static void launch_ahead(const LinLaunch& L, int per, cudaStream_t st) {
+  const unsigned ctas = (unsigned)L.n_items;
+  if (per == 4) ahead::linearize_ahead_kernel<MODE, 4><<<ctas, kSimpleThreads, 0, st>>>(L);
+  else ahead::linearize_ahead_kernel<MODE, 2><<<ctas, kSimpleThreads, 0, st>>>(L);
 }
 
 // Whether a launch needs its status word and work-item counter zeroed: the staged
@@ -1935,12 +2101,18 @@ int launch_linearize(const LinLaunch& L, cudaStream_t st) {
     count_launches(1);
     Lb.status = L.status + 1;  // the second work-item counter
   }
+  const int ahead = ahead_items(L, variant);
   if (split_items(L, variant)) {
     const unsigned ctas = (unsigned)L.n_items * split::kCtas;
     if (L.mode == 0) split::linearize_split_kernel<0><<<ctas, split::kThreads, 0, st>>>(L);
     else if (L.mode == 1) split::linearize_split_kernel<1><<<ctas, split::kThreads, 0, st>>>(L);
     else if (L.mode == 2) split::linearize_split_kernel<2><<<ctas, split::kThreads, 0, st>>>(L);
     else split::linearize_split_kernel<3><<<ctas, split::kThreads, 0, st>>>(L);
+  } else if (ahead > 0) {
+    if (L.mode == 0) launch_ahead<0>(L, ahead, st);
+    else if (L.mode == 1) launch_ahead<1>(L, ahead, st);
+    else if (L.mode == 2) launch_ahead<2>(L, ahead, st);
+    else launch_ahead<3>(L, ahead, st);
   } else if (L.mode != 0) {
     // cost / gradient evaluations use the per-point kernel
     if (L.neighbours == 27) {
