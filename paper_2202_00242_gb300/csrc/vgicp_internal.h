@@ -63,10 +63,10 @@ struct MapSet {
   int32_t* d_status = nullptr;              // 1
   // device: build scratch (kept for rebuilds)
   uint32_t* d_pt_slot = nullptr;  // n_total: build-table slot of each point
-  uint32_t* d_flag = nullptr;     // n_total: voxel id of each point (read at map starts)
+  uint32_t* d_flag = nullptr;     // n_total: bitmap of the voxels' first points
   uint32_t* d_vcount = nullptr;   // n_total: points per voxel
   uint32_t* d_voff = nullptr;     // n_total: voxel at each rank
-  uint32_t* d_vfill = nullptr;    // n_total: first-point flags, counts by rank, list fill
+  uint32_t* d_vfill = nullptr;    // n_total: first points before each bitmap word
   uint32_t* d_plist = nullptr;    // n_total: point lists of the voxels, in rank order
   // kept from one build to the next: the lookup-table slot each voxel occupies,
   // so a rebuild empties just those (every other slot is empty already)
