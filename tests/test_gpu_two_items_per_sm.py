@@ -59,3 +59,20 @@ def test_points_without_a_voxel_and_not_finite(dev):  # noqa: F811
         pts[6] = float("nan")
     _same(a, b, poses)
     assert bool(torch.isfinite(a.execute(poses).out).all())
+
+
+@pytest.mark.parametrize("sizes", [[5000, 3000, 1], [130 * 2048, 9, 9]])
+def test_execution_without_a_status_word(dev, sizes):  # noqa: F811
+    """Where every item has a CTA an execution clears and reads no status word: what an
+    evaluation at a pose that is not finite left there does not reach it."""
+    (a, b), poses = _plans(sizes, 2048)
+    base = torch.tensor(poses, device="cuda")
+    xi = torch.zeros((len(poses), 6), dtype=torch.float64, device="cuda")
+    want = b.execute(poses)
+    for p in (a, b):
+        p.execute(poses)                   # captures
+        xi[0, 0] = float("nan")
+        g, n = p.evaluate(base, xi, mode=2)
+        assert bool(torch.isnan(g).all()) and bool((n == -1).all())
+        got = p.execute(poses)
+        assert torch.equal(got.out, want.out) and torch.equal(got.inliers, want.inliers)
