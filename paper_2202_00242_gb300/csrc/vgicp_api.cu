@@ -117,7 +117,7 @@ int create_set(const int64_t* offsets, int32_t n_maps, double resolution,
   const size_t o_vmask = take(sizeof(uint32_t) * n_maps);
   const size_t o_recs = take(sizeof(float4) * kRecordF4 * n);
   const size_t o_vkeys = take(sizeof(unsigned long long) * n);
-  const size_t o_status = take(sizeof(int32_t));
+  const size_t o_status = take(2 * sizeof(int32_t));
   const size_t o_num_vox = take(sizeof(uint32_t));
   const size_t o_pt_slot = take(sizeof(uint32_t) * n);
   const size_t o_flag = take(sizeof(uint32_t) * n);

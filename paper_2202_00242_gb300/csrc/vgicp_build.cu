@@ -5,8 +5,8 @@
 // Pipeline for a batch of maps built from concatenated clouds (one launch per
 // step for the whole batch):
 //   reset     table slots <- empty: every slot on the first build; afterwards
-//             the lookup-table slots the previous build's voxels occupy (the
-//             build table is left empty by the scatter)
+//             the lookup-table slots the previous build's voxels occupy, by CTAs
+//             of the insertion (the build table is left empty by the scatter)
 //   insert    per point: exact key, open-addressing insert (CAS on the 64-bit
 //             key, bounded linear probe), count, smallest point index
 //   number    first points (the smallest index of their voxel) marked in a
@@ -70,8 +70,14 @@ __device__ __forceinline__ void set_status(int32_t* status, int32_t code) {
   atomicCAS(status, 0, code);
 }
 
+// The status of the insertion becomes the build's; its own word is ready for the next.
+__device__ __forceinline__ void take_status(int32_t* status) {
+  status[0] = status[1];
+  status[1] = 0;
+}
+
 __global__ void init_slots_kernel(Slot* __restrict__ slots, int64_t cap_total, int32_t* status) {
-  if (blockIdx.x == 0 && threadIdx.x == 0) *status = 0;
+  if (blockIdx.x == 0 && threadIdx.x < 2) status[threadIdx.x] = 0;
   for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < cap_total;
        s += (int64_t)gridDim.x * blockDim.x) {
     Slot e;
@@ -82,14 +88,50 @@ __global__ void init_slots_kernel(Slot* __restrict__ slots, int64_t cap_total, i
   }
 }
 
+// Rebuild: empty the lookup-table slots the previous build's voxels occupy
+// (every slot a build claims belongs to one of its voxels, and spill flags are
+// set only on claimed slots), which leaves the tables empty.  (The build table
+// is emptied by the scatter of every build.)
+__device__ void reset_lookup(int cta, int ctas, int64_t n_max, const uint32_t* __restrict__ n_vox,
+                             const uint32_t* __restrict__ lslot_of, VSlot* vslots) {
+  const int64_t V = *n_vox;
+  for (int64_t v = cta * (int64_t)blockDim.x + threadIdx.x; v < V && v < n_max;
+       v += (int64_t)ctas * blockDim.x) {
+    const uint32_t ls = lslot_of[v];
+    if (ls != kNoSlot)
+      asm volatile("st.global.v8.b32 [%0], {%1, %1, %2, %2, %2, %2, %2, %2};" ::"l"(vslots + ls),
+                   "r"(0xFFFFFFFFu), "r"(0u)
+                   : "memory");
+  }
+}
+
+// One CTA in kResetEvery empties lookup slots on a rebuild (a first build passes no CTAs
+// for it): the lookup tables are next written by finalize, and the previous build's
+// voxel count by the numbering, so the reset needs no launch of its own.  Ten maps of
+// 20,000 points rebuilt and ten factors, r 0.25 / 1.0: 118.8 / 104.8 us with a reset
+// kernel, 115.8 / 101.5 so; three maps of 3,000 points 84.7 / 80.2; 500 submaps (25.8M
+// points): insert 598 us with the reset inside, 494 + 114 apart.
+// Errors go to the second status word, which the numbering moves to the first.
+constexpr int kResetEvery = 9;
 __global__ void insert_kernel(const float* __restrict__ pts, int64_t n_total,
                               const int64_t* __restrict__ point_off, int32_t n_maps,
                               const int64_t* __restrict__ slot_base,
                               const uint32_t* __restrict__ cap_mask, float inv_r, double r,
                               int32_t max_probe, Slot* slots, uint32_t* __restrict__ pt_slot,
-                              int32_t* status) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n_total;
-       i += (int64_t)gridDim.x * blockDim.x) {
+                              int32_t* status, int reset_ctas, const uint32_t* __restrict__ n_vox,
+                              const uint32_t* __restrict__ lslot_of, VSlot* vslots) {
+  int cta = blockIdx.x;
+  const int ctas = gridDim.x - reset_ctas;
+  if (reset_ctas > 0) {
+    const int k = cta / kResetEvery;
+    if (cta % kResetEvery == 0 && k < reset_ctas) {
+      reset_lookup(k, reset_ctas, n_total, n_vox, lslot_of, vslots);
+      return;
+    }
+    cta -= min(k + 1, reset_ctas);
+  }
+  for (int64_t i = cta * (int64_t)blockDim.x + threadIdx.x; i < n_total;
+       i += (int64_t)ctas * blockDim.x) {
     const int m = find_map_warp(point_off, n_maps, i);
     const int kx = axis_key_target(__ldg(pts + 3 * i + 0), inv_r, r);
     const int ky = axis_key_target(__ldg(pts + 3 * i + 1), inv_r, r);
@@ -123,28 +165,6 @@ __global__ void insert_kernel(const float* __restrict__ pts, int64_t n_total,
     pt_slot[i] = found;
   }
 }
-
-
-
-// Rebuild: empty the lookup-table slots the previous build's voxels occupy
-// (every slot a build claims belongs to one of its voxels, and spill flags are
-// set only on claimed slots), which leaves the tables empty.  (The build table
-// is emptied by the scatter of every build.)
-__global__ void reset_tables_kernel(int64_t n_max, const uint32_t* __restrict__ n_vox,
-                                    const uint32_t* __restrict__ lslot_of, VSlot* vslots,
-                                    int32_t* status) {
-  if (blockIdx.x == 0 && threadIdx.x == 0) *status = 0;
-  const int64_t V = *n_vox;
-  for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < V && v < n_max;
-       v += (int64_t)gridDim.x * blockDim.x) {
-    const uint32_t ls = lslot_of[v];
-    if (ls != kNoSlot)
-      asm volatile("st.global.v8.b32 [%0], {%1, %1, %2, %2, %2, %2, %2, %2};" ::"l"(vslots + ls),
-                   "r"(0xFFFFFFFFu), "r"(0u)
-                   : "memory");
-  }
-}
-
 
 
 // Per point: append its index to its voxel's list.  The voxel's last point
@@ -1117,7 +1137,8 @@ __global__ void vbase_kernel(int32_t n_maps, int64_t n_total, const int64_t* __r
                              const uint32_t* __restrict__ bitmap,
                              const uint32_t* __restrict__ wscan, uint32_t* __restrict__ vbase,
                              uint32_t* __restrict__ n_vox, const int64_t* __restrict__ vslot_base,
-                             uint32_t* __restrict__ vmask) {
+                             uint32_t* __restrict__ vmask, int32_t* status) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) take_status(status);
   const int m = blockIdx.x * blockDim.x + threadIdx.x;
   if (m <= n_maps)
     map_ranges(m, n_maps, n_total, point_off, bitmap, wscan, vbase, n_vox, vslot_base, vmask);
@@ -1132,8 +1153,9 @@ __global__ void __launch_bounds__(kNumberThreads) number_kernel(
     const uint32_t* bitmap, int64_t n_words, uint32_t* wscan, int32_t n_maps, int64_t n_total,
     const int64_t* __restrict__ point_off, uint32_t* __restrict__ vbase,
     uint32_t* __restrict__ n_vox, const int64_t* __restrict__ vslot_base,
-    uint32_t* __restrict__ vmask) {
+    uint32_t* __restrict__ vmask, int32_t* status) {
   __shared__ uint32_t total;
+  if (threadIdx.x == 0) take_status(status);
   uint32_t carry = 0u;
   for (int64_t w0 = 0; w0 < n_words; w0 += kNumberThreads * kNumberPer) {
     const int64_t a = w0 + (int64_t)threadIdx.x * kNumberPer;
@@ -1228,21 +1250,15 @@ int size_lookup_tables(MapSet* s, cudaStream_t st) {
 
 int launch_build(MapSet* s, const float* points, const float* covs, cudaStream_t st) {
   const int64_t n = s->n_total;
-  // light kernels over voxels (V <= n is on the device): grid-stride, capped grid
-  const int gv = std::min<int>(grid_for(std::max<int64_t>(n, 1), kThreads), device_sm_count() * 8);
   // was_built: the tables hold only the previous build's voxels (a build that
   // stops on an error leaves `built` cleared, so the next one starts over)
   const bool was_built = s->built;
   s->built = false;
-  if (was_built) {
-    // empty the slots of the previous build's voxels
-    reset_tables_kernel<<<gv, kThreads, 0, st>>>(n, s->d_num_voxels, s->d_lslot_of,
-                                                 s->d_vslots, s->d_status);
-  } else {
+  if (!was_built) {
     init_slots_kernel<<<grid_for(s->cap_total, kThreads), kThreads, 0, st>>>(
         s->d_slots, s->cap_total, s->d_status);
+    count_launches(1);
   }
-  count_launches(1);
   if (n == 0) {
     VGICP_CUDA_TRY(cudaMemsetAsync(s->d_num_voxels, 0, sizeof(uint32_t), st));
     VGICP_CUDA_TRY(cudaMemsetAsync(s->d_vbase, 0, sizeof(uint32_t) * (s->n_maps + 1), st));
@@ -1260,9 +1276,11 @@ int launch_build(MapSet* s, const float* points, const float* covs, cudaStream_t
   }
   const float inv_r = (float)(1.0 / s->resolution);
   const int g = grid_for(n, kThreads);
-  insert_kernel<<<g, kThreads, 0, st>>>(points, n, s->d_point_off, s->n_maps, s->d_slot_base,
-                                        s->d_cap_mask, inv_r, s->resolution, s->max_probe,
-                                        s->d_slots, s->d_pt_slot, s->d_status);
+  const int reset = was_built ? std::max(1, g / (kResetEvery - 1)) : 0;
+  insert_kernel<<<g + reset, kThreads, 0, st>>>(
+      points, n, s->d_point_off, s->n_maps, s->d_slot_base, s->d_cap_mask, inv_r, s->resolution,
+      s->max_probe, s->d_slots, s->d_pt_slot, s->d_status + 1, reset, s->d_num_voxels,
+      s->d_lslot_of, s->d_vslots);
   // voxel ids in order of first appearance: first points marked in d_flag, the
   // words' popcounts scanned in d_vfill (both dead afterwards)
   int rc = VGICP_OK;
@@ -1276,14 +1294,14 @@ int launch_build(MapSet* s, const float* points, const float* covs, cudaStream_t
     if (n_words <= kNumberWords) {
       number_kernel<<<1, kNumberThreads, 0, st>>>(bitmap, n_words, wscan, s->n_maps, n,
                                                   s->d_point_off, s->d_vbase, s->d_num_voxels,
-                                                  s->d_vslot_base, vmask);
+                                                  s->d_vslot_base, vmask, s->d_status);
     } else {
       popc_words_kernel<<<grid_for(n_words, kThreads), kThreads, 0, st>>>(bitmap, n_words, wscan);
       rc = launch_exclusive_scan(wscan, wscan, n_words, nullptr, s->d_scan_tmp, nullptr, st);
       if (rc != VGICP_OK) return rc;
       vbase_kernel<<<(s->n_maps + 1 + 127) / 128, 128, 0, st>>>(
           s->n_maps, n, s->d_point_off, bitmap, wscan, s->d_vbase, s->d_num_voxels,
-          s->d_vslot_base, vmask);
+          s->d_vslot_base, vmask, s->d_status);
       count_launches(1);
     }
     assign_ids_kernel<<<g, kThreads, 0, st>>>(bitmap, wscan, n, s->d_pt_slot, s->d_slots,

@@ -60,7 +60,7 @@ struct MapSet {
   uint32_t* d_vmask = nullptr;              // n_maps: lookup-table capacity - 1
   float4* d_recs = nullptr;                 // n_total * 3 (V <= n_total)
   unsigned long long* d_vkeys = nullptr;    // n_total (packed keys by voxel)
-  int32_t* d_status = nullptr;              // 1
+  int32_t* d_status = nullptr;              // 2: the build's, the insertion's
   // device: build scratch (kept for rebuilds)
   uint32_t* d_pt_slot = nullptr;  // n_total: build-table slot of each point
   uint32_t* d_flag = nullptr;     // n_total: bitmap of the voxels' first points
