@@ -476,6 +476,11 @@ int vgicp_plan_evaluate(vgicp_plan* P, const double* base_poses, const double* x
   if (mode < 1 || mode > 3) return set_error(VGICP_ERR_INVALID_ARG, "mode must be 1, 2 or 3");
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   const int32_t number = P->evaluations = P->evaluations % INT32_MAX + 1;  // never 0
+  // an evaluation recorded in a graph keeps its number, so each replay clears the word
+  cudaStreamCaptureStatus recording = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &recording) != cudaSuccess) cudaGetLastError();
+  if (recording != cudaStreamCaptureStatusNone)
+    VGICP_CUDA_TRY(cudaMemsetAsync(P->d_status, 0, sizeof(int32_t), st));
   double* jr = mode >= 2 && xi ? P->d_jr : nullptr;
   const int64_t n = P->n_pairs;
   const dim3 grid((unsigned)((n + kComposeThreads - 1) / kComposeThreads), jr ? 2 : 1);
