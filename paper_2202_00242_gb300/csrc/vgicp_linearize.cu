@@ -551,7 +551,7 @@ __global__ void __launch_bounds__(kThreads, VGICP_MIN_BLOCKS) linearize_tma_kern
     const float* X = reinterpret_cast<const float*>(S.xyz[s] + d.xyz_off);
     const float* C = reinterpret_cast<const float*>(S.cov[s] + d.cov_off);
 
-    // ---- lookup: key, first probe (two 256-bit loads) of every point, resolve ----
+    // ---- lookup: key, first probe (a 256-bit and a 128-bit load) of every point, resolve ----
     int idx[kPtsPerLane];
     int kx[kPtsPerLane], ky[kPtsPerLane], kz[kPtsPerLane];
     bool live[kPtsPerLane];
