@@ -642,7 +642,8 @@ __global__ void __launch_bounds__(32 * W) knn_select_kernel(const Grid G, int32_
       ++n;
     }
   }
-  // the kept values were sorted but for their low bits: neighbours may be swapped
+  // the kept values were sorted but for their low 9 bits: within a step of those any
+  // order is possible.  Two passes of exchanges restore nearly every list.
   auto order2 = [&](int x, int y) {
     const uint32_t lo = min(ord[x], ord[y]), hi = max(ord[x], ord[y]);
     ord[x] = lo;
@@ -652,10 +653,16 @@ __global__ void __launch_bounds__(32 * W) knn_select_kernel(const Grid G, int32_
   for (int x = 0; x + 1 < CAP; x += 2) order2(x, x + 1);
 #pragma unroll
   for (int x = 1; x + 1 < CAP; x += 2) order2(x, x + 1);
+  // Accepted: each of the first k below the one after it, and the k-th below every
+  // later one, by more than the error bound.
+  uint32_t later = ~0u;  // the smallest after the k-th
 #pragma unroll
-  for (int x = 0; x + 1 < CAP; ++x) {  // the first k, and the k-th from the next
+  for (int x = 0; x < CAP; ++x)
+    if (x >= k) later = min(later, ord[x]);
+#pragma unroll
+  for (int x = 0; x + 1 < CAP; ++x) {
     const float lo = __uint_as_float(ord[x] | kSlotBits);
-    const float hi = __uint_as_float(ord[x + 1] & ~kSlotBits);
+    const float hi = __uint_as_float((x + 1 < k ? ord[x + 1] : later) & ~kSlotBits);
     good = good && (x >= k || x + 1 >= n || (hi > lo * kF2Up && hi > kF2Tiny));
   }
   // the others go to the second kernel's list
