@@ -152,7 +152,8 @@ int vgicp_voxelmap_export(const vgicp_map* map, vgicp_stream_t stream, int64_t m
 /* Copies the map's voxel-grouped cloud (the cloud a map-as-source factor reads,
  * Sec. III-F): its n rows with the points of each voxel contiguous and in
  * ascending input index, the voxels in Morton order within chunks of the map's
- * voxels.  points: device n x 3, covs: device n x 6 (either may be NULL);
+ * voxels.  Points without a voxel (VGICP_ERR_KEY_RANGE, VGICP_ERR_HASH_FULL) are
+ * left out, and as many rows of NaN end the cloud.  points: device n x 3, covs: device n x 6 (either may be NULL);
  * asynchronous on stream. */
 int vgicp_voxelmap_grouped_cloud(const vgicp_map* map, vgicp_stream_t stream, float* points,
                                  float* covs);

@@ -172,12 +172,20 @@ __global__ void insert_kernel(const float* __restrict__ pts, int64_t n_total,
 // voxel has read the slot before its own increment) empties the build-table
 // slot, whose sector it has just read: the build table is empty again when the
 // scatter ends, ready for the next build.
+// A point without a voxel (outside the key range, which the build reports) is in no list:
+// it leaves kNoSlot at the end of its map's range of plist, behind the map's last list.
 __global__ void scatter_kernel(int64_t n_total, const uint32_t* __restrict__ pt_slot, Slot* slots,
-                               unsigned long long* bfill, uint32_t* __restrict__ plist) {
+                               unsigned long long* bfill, uint32_t* __restrict__ plist,
+                               const int64_t* __restrict__ point_off, int32_t n_maps,
+                               uint32_t* dropped) {
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n_total;
        i += (int64_t)gridDim.x * blockDim.x) {
     const uint32_t s = pt_slot[i];
-    if (s == kNoSlot) continue;
+    if (s == kNoSlot) {
+      const int m = find_map(point_off, n_maps, i);
+      plist[point_off[m + 1] - 1 - (int64_t)atomicAdd(dropped + m, 1u)] = kNoSlot;
+      continue;
+    }
     // one read of the slot: voxel id and count
     const uint4 w = *reinterpret_cast<const uint4*>(slots + s);
     const uint32_t v = w.z, c = w.w;
@@ -364,10 +372,32 @@ __device__ __forceinline__ void write_record(uint32_t v, uint32_t o, uint32_t c,
   recs[3 * v + 2] = make_float4(q[7], q[8], 0.0f, 0.0f);
 }
 
+// One read of a word that other CTAs may be setting, whose value then stays.  (Rebuild of
+// 500 maps of 50,000 points: 3,091 us so, 3,101 with a relaxed and 3,110 with a volatile
+// load, which the kernel's other loads wait for.)
+__device__ __forceinline__ int32_t read_once(const int32_t* p) {
+  int32_t v;
+  asm("ld.global.b32 %0, [%1];" : "=r"(v) : "l"(p));
+  return v;
+}
+
+// Row d of the grouped cloud without a point: NaN, which is no voxel's.
+__device__ __forceinline__ void empty_row(float* gpts, float* gcovs, int64_t d) {
+  const float nan = __uint_as_float(0x7FFFFFFFu);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) gpts[3 * d + k] = nan;
+#pragma unroll
+  for (int k = 0; k < 6; ++k) gcovs[6 * d + k] = nan;
+}
+
+// Lists lie end to end but for the points without a voxel, which follow their map's last
+// list (or fill the range of a map that has no voxel).  Those exist only after an
+// insertion that reported an error, and only then is a list's length read from its
+// voxel's count instead of the next offset: the read costs a dependent load.
 __global__ void __launch_bounds__(kFinThreads) finalize_kernel(
     int64_t n_max, const uint32_t* __restrict__ n_vox, const float* __restrict__ pts,
     const float* __restrict__ covs, const uint32_t* __restrict__ vorder,
-    const uint32_t* __restrict__ goff,
+    const uint32_t* __restrict__ vcount, const uint32_t* __restrict__ goff,
     uint32_t* __restrict__ plist, float4* __restrict__ recs, float* gpts, float* gcovs,
     const unsigned long long* __restrict__ vkeys, int32_t n_maps,
     const uint32_t* __restrict__ vbase, const int64_t* __restrict__ slot_base,
@@ -377,10 +407,15 @@ __global__ void __launch_bounds__(kFinThreads) finalize_kernel(
   __shared__ int seg_map[2];
   const int64_t V = min((int64_t)*n_vox, n_max);
   const uint32_t total = (uint32_t)n_max;  // end of the last list (goff[V] is not stored)
+  const bool dropped = read_once(status) != 0;
+  if (V == 0)  // no point has a voxel
+    for (int64_t i = blockIdx.x * (int64_t)kFinThreads + threadIdx.x; i < n_max;
+         i += (int64_t)gridDim.x * kFinThreads)
+      empty_row(gpts, gcovs, i);
   for (int64_t r0 = (int64_t)blockIdx.x * kFinThreads; r0 < V; r0 += (int64_t)gridDim.x * kFinThreads) {
     const int64_t r1 = min(V, r0 + kFinThreads);
     // list bounds from consecutive offsets: no dependent load through vorder
-    const uint32_t seg0 = goff[r0];
+    const uint32_t seg0 = r0 > 0 ? goff[r0] : 0u;
     const uint32_t seg1 = r1 < V ? goff[r1] : total;
     const uint32_t len = seg1 - seg0;
     const bool staged = len <= (uint32_t)kFinStage;
@@ -392,7 +427,8 @@ __global__ void __launch_bounds__(kFinThreads) finalize_kernel(
     }
     const uint32_t v = mine ? vorder[r] : 0u;
     const uint32_t o = mine ? goff[r] : 0u;
-    const uint32_t c = mine ? (r + 1 < V ? goff[r + 1] : total) - o : 0u;
+    const uint32_t c =
+        !mine ? 0u : dropped ? vcount[v] : (r + 1 < V ? goff[r + 1] : total) - o;
     // 1. sort the lists by point index
     if (staged) {
       for (uint32_t i = threadIdx.x; i < len; i += kFinThreads) stage[i] = plist[seg0 + i];
@@ -405,9 +441,7 @@ __global__ void __launch_bounds__(kFinThreads) finalize_kernel(
     // 2. gather into the grouped cloud
     const uint32_t* lst = staged ? stage : plist + seg0;
     for (uint32_t i = threadIdx.x; i < len; i += kFinThreads) {
-      // (a point without a voxel, which the build reports, leaves a gap behind its map's
-      // last list, whatever it holds)
-      const int64_t j = min(lst[i], total - 1u);
+      const int64_t j = min(lst[i], total - 1u);  // (kNoSlot: the row is emptied below)
       const float x = __ldg(pts + 3 * j), y = __ldg(pts + 3 * j + 1), z = __ldg(pts + 3 * j + 2);
       const float2* cv = reinterpret_cast<const float2*>(covs + 6 * j);
       const float2 c0 = __ldg(cv), c1 = __ldg(cv + 1), c2 = __ldg(cv + 2);
@@ -420,6 +454,9 @@ __global__ void __launch_bounds__(kFinThreads) finalize_kernel(
       gc[1] = c1;
       gc[2] = c2;
     }
+    if (dropped)
+      for (uint32_t i = threadIdx.x; i < len; i += kFinThreads)
+        if (lst[i] == kNoSlot) empty_row(gpts, gcovs, (int64_t)seg0 + i);
     __syncthreads();  // the CTA's global writes are visible to the CTA after this
     // 3. sums from the grouped copy (plain loads: written by this kernel)
     if (mine) {
@@ -470,12 +507,12 @@ __device__ __forceinline__ void add_lane(float* hi, float* lo, bool& exact, int 
 // points 19 / 18 us (2.0), 20 / 28 (5.7), 19 / 55 (11), 21 / 148 (23), 49 / 1554 (91);
 // 20 maps of 40,000 52 / 66 (11); 100 maps of 50,000 252 / 230 (3.8), 226 / 212 (8.1),
 // 233 / 314 (15), 322 / 781 (33).  More registers (80 against 56) cost it the large
-// sets of short lists.
+// sets of short lists (six CTAs per SM asked for: the compiler takes 96 otherwise).
 constexpr uint32_t kFinSerial = 64;
-__global__ void __launch_bounds__(kFinThreads) finalize_long_kernel(
+__global__ void __launch_bounds__(kFinThreads, 6) finalize_long_kernel(
     int64_t n_max, const uint32_t* __restrict__ n_vox, const float* __restrict__ pts,
     const float* __restrict__ covs, const uint32_t* __restrict__ vorder,
-    const uint32_t* __restrict__ goff,
+    const uint32_t* __restrict__ vcount, const uint32_t* __restrict__ goff,
     uint32_t* __restrict__ plist, float4* __restrict__ recs, float* gpts, float* gcovs,
     const unsigned long long* __restrict__ vkeys, int32_t n_maps,
     const uint32_t* __restrict__ vbase, const int64_t* __restrict__ slot_base,
@@ -485,6 +522,11 @@ __global__ void __launch_bounds__(kFinThreads) finalize_long_kernel(
   __shared__ uint32_t list_at[kFinThreads];  // first entry of each list, in the segment
   const int64_t V = min((int64_t)*n_vox, n_max);
   const uint32_t total = (uint32_t)n_max;  // end of the last list (goff[V] is not stored)
+  const bool dropped = read_once(status) != 0;
+  if (V == 0)  // no point has a voxel
+    for (int64_t i = blockIdx.x * (int64_t)kFinThreads + threadIdx.x; i < n_max;
+         i += (int64_t)gridDim.x * kFinThreads)
+      empty_row(gpts, gcovs, i);
   const uint32_t avg = (uint32_t)(n_max / max((int64_t)1, V));
   int R = kFinThreads;
   while (R > 4 && (uint32_t)R * avg > 512u) R >>= 1;
@@ -492,15 +534,16 @@ __global__ void __launch_bounds__(kFinThreads) finalize_long_kernel(
   const int lane = threadIdx.x & 31, part = (int)threadIdx.x & (per - 1);
   for (int64_t r0 = (int64_t)blockIdx.x * R; r0 < V; r0 += (int64_t)gridDim.x * R) {
     const int64_t r1 = min(V, r0 + R);
-    const uint32_t seg0 = goff[r0];
+    const uint32_t seg0 = r0 > 0 ? goff[r0] : 0u;
     const uint32_t seg1 = r1 < V ? goff[r1] : total;
     const uint32_t len = seg1 - seg0;
     const bool staged = len <= (uint32_t)kFinStage;
     const int64_t r = r0 + (int)threadIdx.x / per;
     const bool ours = r < r1, mine = ours && part == 0;
-    const uint32_t v = mine ? vorder[r] : 0u;
+    const uint32_t v = mine || (ours && dropped) ? vorder[r] : 0u;
     const uint32_t o = ours ? goff[r] : 0u;
-    const uint32_t c = ours ? (r + 1 < V ? goff[r + 1] : total) - o : 0u;
+    const uint32_t c =
+        !ours ? 0u : dropped ? vcount[v] : (r + 1 < V ? goff[r + 1] : total) - o;
     if (staged) {
       for (uint32_t i = threadIdx.x; i < len; i += kFinThreads) stage[i] = plist[seg0 + i];
       if (mine) list_at[r - r0] = o - seg0;
@@ -510,12 +553,12 @@ __global__ void __launch_bounds__(kFinThreads) finalize_long_kernel(
     __syncthreads();
     for (uint32_t i = threadIdx.x; i < len; i += kFinThreads) {
       const uint32_t id = staged ? stage[i] : plist[seg0 + i];
-      const int64_t j = min(id, total - 1u);  // (see above)
+      const int64_t j = min(id, total - 1u);  // (kNoSlot: the row is emptied below)
       const float x = __ldg(pts + 3 * j), y = __ldg(pts + 3 * j + 1), z = __ldg(pts + 3 * j + 2);
       const float2* cv = reinterpret_cast<const float2*>(covs + 6 * j);
       const float2 c0 = __ldg(cv), c1 = __ldg(cv + 1), c2 = __ldg(cv + 2);
       int64_t d = (int64_t)seg0 + i;
-      if (staged) {
+      if (staged && id != kNoSlot) {
         int q = 0, end = (int)(r1 - r0);  // the entry's list: the last with list_at <= i
         while (end - q > 1) {
           const int mid = (q + end) >> 1;
@@ -535,6 +578,10 @@ __global__ void __launch_bounds__(kFinThreads) finalize_long_kernel(
       gc[1] = c1;
       gc[2] = c2;
     }
+    if (dropped)
+      for (uint32_t i = threadIdx.x; i < len; i += kFinThreads)
+        if ((staged ? stage[i] : plist[seg0 + i]) == kNoSlot)
+          empty_row(gpts, gcovs, (int64_t)seg0 + i);
     __syncthreads();  // the CTA's global writes are visible to the CTA after this
     float hi[9], lo[9], q[9];
 #pragma unroll
@@ -1114,17 +1161,19 @@ __global__ void assign_ids_kernel(const uint32_t* __restrict__ bitmap,
 }
 
 // vbase[m] = voxels of the maps before m; vbase[n_maps] and *n_vox = all.  With vmask
-// (a rebuild) also each map's lookup-table mask.
+// (a rebuild) also each map's lookup-table mask.  The scatter's counters start at zero.
 __device__ __forceinline__ void map_ranges(int m, int32_t n_maps, int64_t n_total,
                                            const int64_t* __restrict__ point_off,
                                            const uint32_t* bitmap, const uint32_t* wscan,
                                            uint32_t* __restrict__ vbase,
                                            uint32_t* __restrict__ n_vox,
                                            const int64_t* __restrict__ vslot_base,
-                                           uint32_t* __restrict__ vmask) {
+                                           uint32_t* __restrict__ vmask,
+                                           uint32_t* __restrict__ dropped) {
   const uint32_t v =
       first_rank(bitmap, wscan, (uint32_t)(m < n_maps ? point_off[m] : n_total));
   vbase[m] = v;
+  if (m < n_maps) dropped[m] = 0u;
   if (m == n_maps) {
     *n_vox = v;
   } else if (vmask) {
@@ -1137,11 +1186,13 @@ __global__ void vbase_kernel(int32_t n_maps, int64_t n_total, const int64_t* __r
                              const uint32_t* __restrict__ bitmap,
                              const uint32_t* __restrict__ wscan, uint32_t* __restrict__ vbase,
                              uint32_t* __restrict__ n_vox, const int64_t* __restrict__ vslot_base,
-                             uint32_t* __restrict__ vmask, int32_t* status) {
+                             uint32_t* __restrict__ vmask, int32_t* status,
+                             uint32_t* __restrict__ dropped) {
   if (blockIdx.x == 0 && threadIdx.x == 0) take_status(status);
   const int m = blockIdx.x * blockDim.x + threadIdx.x;
   if (m <= n_maps)
-    map_ranges(m, n_maps, n_total, point_off, bitmap, wscan, vbase, n_vox, vslot_base, vmask);
+    map_ranges(m, n_maps, n_total, point_off, bitmap, wscan, vbase, n_vox, vslot_base, vmask,
+               dropped);
 }
 
 // The words' popcounts scanned and the maps' ranges, by one CTA: five launches in one
@@ -1153,7 +1204,7 @@ __global__ void __launch_bounds__(kNumberThreads) number_kernel(
     const uint32_t* bitmap, int64_t n_words, uint32_t* wscan, int32_t n_maps, int64_t n_total,
     const int64_t* __restrict__ point_off, uint32_t* __restrict__ vbase,
     uint32_t* __restrict__ n_vox, const int64_t* __restrict__ vslot_base,
-    uint32_t* __restrict__ vmask, int32_t* status) {
+    uint32_t* __restrict__ vmask, int32_t* status, uint32_t* __restrict__ dropped) {
   __shared__ uint32_t total;
   if (threadIdx.x == 0) take_status(status);
   uint32_t carry = 0u;
@@ -1175,7 +1226,8 @@ __global__ void __launch_bounds__(kNumberThreads) number_kernel(
     __syncthreads();  // the CTA's words are visible to it; `total` may be rewritten
   }
   for (int m = threadIdx.x; m <= n_maps; m += kNumberThreads)
-    map_ranges(m, n_maps, n_total, point_off, bitmap, wscan, vbase, n_vox, vslot_base, vmask);
+    map_ranges(m, n_maps, n_total, point_off, bitmap, wscan, vbase, n_vox, vslot_base, vmask,
+               dropped);
 }
 
 // One thread per element (no grid-stride cap): CTAs are dispatched roughly in
@@ -1294,14 +1346,15 @@ int launch_build(MapSet* s, const float* points, const float* covs, cudaStream_t
     if (n_words <= kNumberWords) {
       number_kernel<<<1, kNumberThreads, 0, st>>>(bitmap, n_words, wscan, s->n_maps, n,
                                                   s->d_point_off, s->d_vbase, s->d_num_voxels,
-                                                  s->d_vslot_base, vmask, s->d_status);
+                                                  s->d_vslot_base, vmask, s->d_status,
+                                                  s->d_dropped);
     } else {
       popc_words_kernel<<<grid_for(n_words, kThreads), kThreads, 0, st>>>(bitmap, n_words, wscan);
       rc = launch_exclusive_scan(wscan, wscan, n_words, nullptr, s->d_scan_tmp, nullptr, st);
       if (rc != VGICP_OK) return rc;
       vbase_kernel<<<(s->n_maps + 1 + 127) / 128, 128, 0, st>>>(
           s->n_maps, n, s->d_point_off, bitmap, wscan, s->d_vbase, s->d_num_voxels,
-          s->d_vslot_base, vmask, s->d_status);
+          s->d_vslot_base, vmask, s->d_status, s->d_dropped);
       count_launches(1);
     }
     assign_ids_kernel<<<g, kThreads, 0, st>>>(bitmap, wscan, n, s->d_pt_slot, s->d_slots,
@@ -1326,7 +1379,8 @@ int launch_build(MapSet* s, const float* points, const float* covs, cudaStream_t
                                             : launch_sort<1, 1024>(s, vorder, bfill, st);
   if (rc != VGICP_OK) return rc;
   VGICP_CUDA_TRY(cudaGetLastError());
-  scatter_kernel<<<g, kThreads, 0, st>>>(n, s->d_pt_slot, s->d_slots, bfill, s->d_plist);
+  scatter_kernel<<<g, kThreads, 0, st>>>(n, s->d_pt_slot, s->d_slots, bfill, s->d_plist,
+                                         s->d_point_off, s->n_maps, s->d_dropped);
   if (!was_built) {  // empty the whole lookup region and set the masks
     int64_t max_cap = 16;
     for (int32_t m = 0; m < s->n_maps; ++m)
@@ -1342,7 +1396,7 @@ int launch_build(MapSet* s, const float* points, const float* covs, cudaStream_t
   const auto finalize =
       s->avg_list > 10 || n < 500000 ? finalize_long_kernel : finalize_kernel;
   finalize<<<g, kFinThreads, 0, st>>>(
-      n, s->d_num_voxels, points, covs, vorder, s->d_goff, s->d_plist, s->d_recs,
+      n, s->d_num_voxels, points, covs, vorder, s->d_vcount, s->d_goff, s->d_plist, s->d_recs,
       s->d_gpts, s->d_gcovs, s->d_vkeys, s->n_maps, s->d_vbase, s->d_vslot_base, s->d_vmask,
       s->max_probe, s->d_vslots, s->d_lslot_of, s->d_status);
   VGICP_CUDA_TRY(cudaGetLastError());
