@@ -30,7 +30,7 @@ struct vgicp_plan {
   int32_t variant = 0, item = 0, grid = 0;  // current launch shape
   int64_t n_items = 0;
   int64_t items_cap = 0;
-  int32_t evaluations = 0;       // differentiable evaluations so far (numbers them)
+  int32_t evaluations = 0;       // number of the last differentiable evaluation (0: none)
   // device
   char* d_block = nullptr;
   PairDesc* d_pd = nullptr;
@@ -475,11 +475,14 @@ int vgicp_plan_evaluate(vgicp_plan* P, const double* base_poses, const double* x
   if (!P || !base_poses || !out) return set_error(VGICP_ERR_INVALID_ARG, "null plan, poses or out");
   if (mode < 1 || mode > 3) return set_error(VGICP_ERR_INVALID_ARG, "mode must be 1, 2 or 3");
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  const int32_t number = P->evaluations = P->evaluations % INT32_MAX + 1;  // never 0
-  // an evaluation recorded in a graph keeps its number, so each replay clears the word
+  // numbers 2, 3, ...: 0 is a clear word, 1 what an expired wait of an execution leaves
+  const int32_t number = P->evaluations = P->evaluations < 2 || P->evaluations == INT32_MAX
+                                              ? 2 : P->evaluations + 1;
+  // an evaluation recorded in a graph keeps its number, so each replay clears the word;
+  // so does the first evaluation, and the one whose number comes round again
   cudaStreamCaptureStatus recording = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(st, &recording) != cudaSuccess) cudaGetLastError();
-  if (recording != cudaStreamCaptureStatusNone)
+  if (recording != cudaStreamCaptureStatusNone || number == 2)
     VGICP_CUDA_TRY(cudaMemsetAsync(P->d_status, 0, sizeof(int32_t), st));
   double* jr = mode >= 2 && xi ? P->d_jr : nullptr;
   const int64_t n = P->n_pairs;
