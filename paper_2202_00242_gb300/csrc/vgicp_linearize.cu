@@ -871,34 +871,36 @@ __global__ void __launch_bounds__(kSimpleThreads, simple_ctas(NEIGH, MODE))
         const float qz = fmaf(P.R[6], x, fmaf(P.R[7], y, fmaf(P.R[8], z, P.t[2])));
         // Exact key.  y = q / r is split into the nearest integer n and f = y - n (exact)
         // by adding and subtracting 1.5 * 2^23; floor(y) = n - (f < 0), and a face is
-        // near when |f| is below the margin of source_key.  |y| >= 2^22 (and NaN) lies
-        // outside the key range.
+        // near when |f| is below the margin of source_key.  From |y| = 2^22 on the split
+        // fails, and float32 may be further off than the key range is wide: binary64.  A
+        // NaN is no voxel's.
         int kx, ky, kz;
         {
           const float m = fmaf(fabsf(x) + fabsf(y) + fabsf(z) + P.tmax, md.margin_scale,
                                1.1920928955078125e-7f);
           const float yx = qx * md.inv_r, yy = qy * md.inv_r, yz = qz * md.inv_r;
-          constexpr float kMagic = 12582912.0f;
+          constexpr float kMagic = 12582912.0f, kFar = 4194304.0f;
           constexpr int kMagicBits = 0x4B400000;
           const float nx = yx + kMagic, ny = yy + kMagic, nz = yz + kMagic;
           const float fx = yx - (nx - kMagic), fy = yy - (ny - kMagic), fz = yz - (nz - kMagic);
           kx = __float_as_int(nx) - kMagicBits + (__float_as_int(fx) >> 31);
           ky = __float_as_int(ny) - kMagicBits + (__float_as_int(fy) >> 31);
           kz = __float_as_int(nz) - kMagicBits + (__float_as_int(fz) >> 31);
-          const bool inside =
-              fabsf(yx) < 4194304.0f && fabsf(yy) < 4194304.0f && fabsf(yz) < 4194304.0f;
+          const bool inside = fabsf(yx) < kFar && fabsf(yy) < kFar && fabsf(yz) < kFar;
           const bool ax = fabsf(fx) < m, ay = fabsf(fy) < m, az = fabsf(fz) < m;
-          if (inside && (ax | ay | az)) {  // the binary64 path reads r from shared memory
-            MapDesc mr;
-            mr.r = ic.r;
-            if (ax) kx = axis_key_f64(ic.pd, mr, 0, x, y, z);
-            if (ay) ky = axis_key_f64(ic.pd, mr, 1, x, y, z);
-            if (az) kz = axis_key_f64(ic.pd, mr, 2, x, y, z);
+          if (!inside || (ax | ay | az)) {  // the binary64 path reads r from shared memory
+            if (m != m) {
+              kx = 2 * kKeyMin;  // no neighbour is in range either
+            } else {
+              MapDesc mr;
+              mr.r = ic.r;
+              if (ax || !inside) kx = axis_key_f64(ic.pd, mr, 0, x, y, z);
+              if (ay || !inside) ky = axis_key_f64(ic.pd, mr, 1, x, y, z);
+              if (az || !inside) kz = axis_key_f64(ic.pd, mr, 2, x, y, z);
+            }
           }
-          if (!inside) {
-            if (DBG) source_key(P, ic.pd, md_of_item(md, ic.r), x, y, z, qx, qy, qz, kx, ky, kz);
-            else kx = 2 * kKeyMin;  // no neighbour is in range either
-          }
+          if (DBG && !inside)
+            source_key(P, ic.pd, md_of_item(md, ic.r), x, y, z, qx, qy, qz, kx, ky, kz);
         }
         if (DBG && L.qkey_out) {
           L.qkey_out[3 * (b0 + i) + 0] = kx;
