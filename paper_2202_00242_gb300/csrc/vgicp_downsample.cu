@@ -9,8 +9,8 @@
 // order; a point more than `split` away from it in time goes to the voxel's
 // second output voxel.  Output voxels are numbered in order of first
 // appearance, cloud by cloud; each holds the mean of its points' positions and
-// times, the binary64 mean rounded to float32 (exact double-float sums, else
-// binary64 sums in index order).
+// times, the binary64 mean rounded to float32 (of the double-float sum in index order
+// where that is exact, else of the binary64 sum in that order).
 //
 //   insert   per point: exact key, CAS into the cloud's table, first index
 //   group    per point: sub-voxel from the first point's time; first index and
@@ -19,9 +19,9 @@
 //   scatter  the points of each group, contiguous; beside it, the scan of the
 //            bitmap's words (a group's output voxel is the number of first points
 //            before its own) and the clouds' output offsets
-//   finalize per first point: exact sums of its group's list, means.  The sums are
-//            exact in any order, so the lists are not sorted (only a group whose
-//            partial sums round is, for the binary64 sum in index order)
+//   finalize per first point: exact sums of its group's list, means.  Short lists are
+//            sorted; a long one is summed by a warp as it comes, and sorted only if its
+//            sums round in that order, or if another order's could give another mean
 // Six launches, one copy in and one out: a sweep of 60,000 points is bound by their
 // latency and the host's (290 -> 215 us a call, of which the kernels take 33 us; before,
 // 14 kernels, three fills and five copies, 65 us, and a thread per voxel that sorted
@@ -301,9 +301,36 @@ __device__ __forceinline__ void ds_add_lane(float* hi, float* lo, bool& exact, i
   }
 }
 
+// Whether every value within `error` of s has the mean q = RN32(s / n) (m: s / n in
+// binary64): the distance of m to the ends of what rounds to q, in float32.
+__device__ __forceinline__ bool mean_is_certain(double m, float q, float error_of_mean) {
+  const uint32_t b = __float_as_uint(q) & 0x7FFFFFFFu;
+  if (b < (27u << 23) || b >= 0x7F800000u) return false;
+  const float spacing = __uint_as_float((b & 0x7F800000u) - (23u << 23));
+  const float half = (b & 0x007FFFFFu) ? 0.5f * spacing : 0.25f * spacing;  // a power of two: below
+  const float off = fabsf((float)(m - (double)q));
+  return half - off > error_of_mean + 0x1p-22f * spacing;
+}
+
+// Whether c values have the same binary64 sum in every order, an exact one: every partial
+// sum is a multiple of the last bit of the smallest above zero (as bits, less one), and
+// below 2^53 of them.
+__device__ __forceinline__ bool any_order(uint32_t c, float largest, uint32_t smallest) {
+  if (largest == 0.f) return true;
+  const int top = max((int)(__float_as_uint(largest) >> 23), 1);
+  const int low = max((int)((smallest + 1u) >> 23), 1);
+  return top < 255 && top - low + 32 - __clz((int)(c - 1u)) <= 29;
+}
+
 // One lane per point; the lanes of first points take their group's list, lists
-// longer than kSerial the whole warp.
-constexpr uint32_t kSerial = 8;
+// longer than kSerial the whole warp.  Lists are in the order in which their points came,
+// so what depends on the order of a sum must not reach the output.  A sum in double-float
+// that is exact in this order is the true one; the sum in index order, exact or in
+// binary64, is within c^2 max |v| 2^-53 of it, and nearly always has the same mean.
+// The kernel, sweeps of 60,000 points at 0.25 / 1.0 m: 16 / 30 us, of 250,000: 42 / 92;
+// with every sum taken in the order of its list 17 / 34 and 37 / 110; with the smallest
+// magnitude of every long list taken along with its sums 15 / 37 and 44 / 123.
+constexpr uint32_t kSerial = 8;  // as many as the sorting network takes
 __global__ void __launch_bounds__(kThreads) ds_finalize_kernel(
     int64_t n, const uint32_t* __restrict__ bitmap, const uint32_t* __restrict__ wscan,
     const uint32_t* __restrict__ pt_group, const DsGroup* __restrict__ groups,
@@ -319,63 +346,130 @@ __global__ void __launch_bounds__(kThreads) ds_finalize_kernel(
     at = g.z - g.y;
   }
   float hi[4] = {0.f, 0.f, 0.f, 0.f}, lo[4] = {0.f, 0.f, 0.f, 0.f};
+  float largest[4] = {0.f, 0.f, 0.f, 0.f};
   bool exact = true;
-  auto add = [&](uint32_t entry, float* h, float* l, bool& ex) {
-    const int64_t j = list[entry];
-    df_add(h[0], l[0], pts[3 * j], ex);
-    df_add(h[1], l[1], pts[3 * j + 1], ex);
-    df_add(h[2], l[2], pts[3 * j + 2], ex);
-    if (times) df_add(h[3], l[3], times[j], ex);
-  };
-  if (c <= kSerial)
-    for (uint32_t a = 0; a < c; ++a) add(at + a, hi, lo, exact);
   for (uint32_t todo = __ballot_sync(0xFFFFFFFFu, c > kSerial); todo; todo &= todo - 1u) {
     const int b = __ffs(todo) - 1;
     const uint32_t ab = __shfl_sync(0xFFFFFFFFu, at, b), cb = __shfl_sync(0xFFFFFFFFu, c, b);
-    float h[4] = {0.f, 0.f, 0.f, 0.f}, l[4] = {0.f, 0.f, 0.f, 0.f};
+    float h[4] = {0.f, 0.f, 0.f, 0.f}, l[4] = {0.f, 0.f, 0.f, 0.f}, g[4] = {0.f, 0.f, 0.f, 0.f};
     bool ex = true;
-    for (uint32_t a = lane; a < cb; a += 32) add(ab + a, h, l, ex);
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) ds_add_lane(h, l, ex, d);
-    if (lane == b) {
+    for (uint32_t a = lane; a < cb; a += 32) {
+      const int64_t j = list[ab + a];
+      const float f[4] = {pts[3 * j], pts[3 * j + 1], pts[3 * j + 2], times ? times[j] : 0.f};
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
+        if (k == 3 && !times) break;
+        df_add(h[k], l[k], f[k], ex);
+        g[k] = fmaxf(g[k], fabsf(f[k]));
+      }
+    }
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) ds_add_lane(h, l, ex, d);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const uint32_t m = __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(g[k]));
+      if (lane == b) {
         hi[k] = h[k];
         lo[k] = l[k];
+        largest[k] = __uint_as_float(m);
       }
-      exact = ex;
+    }
+    if (lane == b) exact = ex;
+  }
+  // A long list's mean is certain if no sum within the error rounds to another, or (the
+  // quotient on a midpoint, mostly) if every order has the same sum.
+  const double N = (double)c, y = __drcp_rn(N);
+  float mean[4];
+  bool certain = exact && c > kSerial, same_mean = certain;
+  if (certain) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const double m = div_rn(__dadd_rn((double)hi[k], (double)lo[k]), N, y);
+      mean[k] = __double2float_rn(m);
+      same_mean = same_mean && (largest[k] == 0.f ||
+                                mean_is_certain(m, mean[k], (float)c * largest[k] * 0x1p-52f));
+    }
+  }
+  for (uint32_t todo = __ballot_sync(0xFFFFFFFFu, certain && !same_mean); todo; todo &= todo - 1u) {
+    const int b = __ffs(todo) - 1;
+    const uint32_t ab = __shfl_sync(0xFFFFFFFFu, at, b), cb = __shfl_sync(0xFFFFFFFFu, c, b);
+    uint32_t smallest[4] = {kNone, kNone, kNone, kNone};  // above zero, as bits less one
+    for (uint32_t a = lane; a < cb; a += 32) {
+      const int64_t j = list[ab + a];
+      const float f[4] = {pts[3 * j], pts[3 * j + 1], pts[3 * j + 2], times ? times[j] : 0.f};
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        smallest[k] = min(smallest[k], (__float_as_uint(f[k]) & 0x7FFFFFFFu) - 1u);
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const uint32_t m = __reduce_min_sync(0xFFFFFFFFu, smallest[k]);
+      if (lane == b) certain = certain && any_order(c, largest[k], m);
     }
   }
   if (!mine) return;
-  double s[4];
-  if (exact) {
+  if (!certain) {  // in ascending point index
+    double s[4] = {0.0, 0.0, 0.0, 0.0};
+    exact = true;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) s[k] = __dadd_rn((double)hi[k], (double)lo[k]);
-  } else {  // binary64 sums in ascending point index
-    uint32_t* L = list + at;
-    for (uint32_t a = 1; a < c; ++a) {
-      const uint32_t x = L[a];
-      int b = (int)a - 1;
-      while (b >= 0 && L[b] > x) {
-        L[b + 1] = L[b];
-        --b;
-      }
-      L[b + 1] = x;
-    }
+    for (int k = 0; k < 4; ++k) hi[k] = lo[k] = 0.f;
+    auto add_exact = [&](int64_t j) {
 #pragma unroll
-    for (int k = 0; k < 4; ++k) s[k] = 0.0;
-    for (uint32_t a = 0; a < c; ++a) {
-      const int64_t j = L[a];
+      for (int k = 0; k < 3; ++k) df_add(hi[k], lo[k], pts[3 * j + k], exact);
+      if (times) df_add(hi[3], lo[3], times[j], exact);
+    };
+    auto add_64 = [&](int64_t j) {
 #pragma unroll
       for (int k = 0; k < 3; ++k) s[k] = __dadd_rn(s[k], (double)pts[3 * j + k]);
       if (times) s[3] = __dadd_rn(s[3], (double)times[j]);
+    };
+    if (c <= kSerial) {
+      uint32_t e[kSerial];
+#pragma unroll
+      for (int a = 0; a < (int)kSerial; ++a) e[a] = a < (int)c ? list[at + a] : kNone;
+      // odd-even merge network
+      constexpr int kPairs[19][2] = {{0, 1}, {2, 3}, {4, 5}, {6, 7}, {0, 2}, {1, 3}, {4, 6},
+                                     {5, 7}, {1, 2}, {5, 6}, {0, 4}, {1, 5}, {2, 6}, {3, 7},
+                                     {2, 4}, {3, 5}, {1, 2}, {3, 4}, {5, 6}};
+#pragma unroll
+      for (int q = 0; q < 19; ++q) {
+        uint32_t &l = e[kPairs[q][0]], &h = e[kPairs[q][1]];
+        const uint32_t low = min(l, h);
+        h = max(l, h);
+        l = low;
+      }
+#pragma unroll
+      for (int a = 0; a < (int)kSerial; ++a)
+        if (a < (int)c) add_exact(e[a]);
+      if (!exact)
+#pragma unroll
+        for (int a = 0; a < (int)kSerial; ++a)
+          if (a < (int)c) add_64(e[a]);
+    } else {
+      uint32_t* L = list + at;
+      for (uint32_t a = 1; a < c; ++a) {
+        const uint32_t x = L[a];
+        int b = (int)a - 1;
+        while (b >= 0 && L[b] > x) {
+          L[b + 1] = L[b];
+          --b;
+        }
+        L[b + 1] = x;
+      }
+      for (uint32_t a = 0; a < c; ++a) add_exact(L[a]);
+      if (!exact)
+        for (uint32_t a = 0; a < c; ++a) add_64(L[a]);
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      if (exact) s[k] = __dadd_rn((double)hi[k], (double)lo[k]);
+      mean[k] = __double2float_rn(div_rn(s[k], N, y));
     }
   }
   const int64_t v = rank_of(bitmap, wscan, i);
-  const double N = (double)c, y = __drcp_rn(N);
 #pragma unroll
-  for (int k = 0; k < 3; ++k) out_pts[3 * v + k] = __double2float_rn(div_rn(s[k], N, y));
-  if (out_times) out_times[v] = __double2float_rn(div_rn(s[3], N, y));
+  for (int k = 0; k < 3; ++k) out_pts[3 * v + k] = mean[k];
+  if (out_times) out_times[v] = mean[3];
   if (out_counts) out_counts[v] = (int32_t)c;
 }
 
