@@ -292,12 +292,21 @@ __device__ __forceinline__ int map_of_rank(const uint32_t* __restrict__ vbase, i
   return lo;
 }
 
+// Least magnitude above zero among covariance entries off the diagonal (f: a point, then
+// xx xy xz yy yz zz), as twice the bits less one: zeros last.
+__device__ __forceinline__ uint32_t least_off_diagonal(uint32_t low, const float* f) {
+  const uint32_t xy = 2u * __float_as_uint(f[4]) - 1u, xz = 2u * __float_as_uint(f[5]) - 1u,
+                 yz = 2u * __float_as_uint(f[7]) - 1u;
+  return min(min(low, xy), min(xz, yz));
+}
+
 // Exact sums of list entries o + first, o + first + step, ... < o + c of the grouped
 // cloud (plain loads: written by the caller's kernel), in double-float: hi + lo stays
 // the exact sum while each TwoSum error adds exactly to lo (checked).
+template <bool LOW>
 __device__ __forceinline__ void sum_entries(const float* gpts, const float* gcovs, uint32_t o,
                                             uint32_t c, uint32_t first, uint32_t step, float* hi,
-                                            float* lo, bool& exact) {
+                                            float* lo, bool& exact, uint32_t& low) {
   for (uint32_t a = first; a < c; a += step) {
     const int64_t d = (int64_t)o + a;
     float f[9];
@@ -315,26 +324,52 @@ __device__ __forceinline__ void sum_entries(const float* gpts, const float* gcov
       hi[k] = t;
       lo[k] = u;
     }
+    if (LOW) low = least_off_diagonal(low, f);
   }
 }
 
-// The record of voxel v (c points at o of the grouped cloud) from its sums; q: the
-// means of the nine components.
-__device__ __forceinline__ void write_record(uint32_t v, uint32_t o, uint32_t c, float* hi,
-                                             float* lo, bool exact, const float* gpts,
-                                             const float* gcovs, float4* __restrict__ recs,
-                                             float* q) {
+// A binary64 sum in the two words of (hi, lo).
+__device__ __forceinline__ void put_sum64(double s, float& hi, float& lo) {
+  hi = __int_as_float(__double2hiint(s));
+  lo = __int_as_float(__double2loint(s));
+}
+__device__ __forceinline__ double get_sum64(float hi, float lo) {
+  return __hiloint2double(__float_as_int(hi), __float_as_int(lo));
+}
+
+// The binary64 sums of a list in ascending point index (the grouped order), where those in
+// double-float are not exact (rare: large dynamic range).
+__device__ __forceinline__ void sum_entries64(const float* gpts, const float* gcovs, uint32_t o,
+                                              uint32_t c, float* hi, float* lo) {
+  double sum[9];
 #pragma unroll
-  for (int k = 0; k < 9; ++k) {  // hi = RN(hi + lo), lo = the exact remainder
-    float t, e;
-    two_sum(hi[k], lo[k], t, e);
-    hi[k] = t;
-    lo[k] = e;
+  for (int k = 0; k < 9; ++k) sum[k] = 0.0;
+  for (uint32_t a = 0; a < c; ++a) {
+    const int64_t d = (int64_t)o + a;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) sum[k] = __dadd_rn(sum[k], (double)gpts[3 * d + k]);
+#pragma unroll
+    for (int k = 0; k < 6; ++k) sum[3 + k] = __dadd_rn(sum[3 + k], (double)gcovs[6 * d + k]);
   }
+#pragma unroll
+  for (int k = 0; k < 9; ++k) put_sum64(sum[k], hi[k], lo[k]);
+}
+
+// The record of voxel v (c points) from its sums: exact ones in double-float, else (words
+// of) the binary64 ones; q: the means of the nine components.
+__device__ __forceinline__ void write_record(uint32_t v, uint32_t c, float* hi, float* lo,
+                                             bool exact, float4* __restrict__ recs, float* q) {
   // q = RN32(RN64(sum / N)) per component: from the exact float pair in
   // float32 where certified, else (rare) from the binary64 definition
   uint32_t need64 = exact ? 0u : 0x1FFu;
   if (exact) {
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {  // hi = RN(hi + lo), lo = the exact remainder
+      float t, e;
+      two_sum(hi[k], lo[k], t, e);
+      hi[k] = t;
+      lo[k] = e;
+    }
     const float rN = __frcp_rn((float)c);
 #pragma unroll
     for (int k = 0; k < 9; ++k) {
@@ -344,28 +379,15 @@ __device__ __forceinline__ void write_record(uint32_t v, uint32_t o, uint32_t c,
     }
   }
   if (need64) {
-    double sum[9];
-    if (exact) {
-#pragma unroll
-      for (int k = 0; k < 9; ++k) sum[k] = __dadd_rn((double)hi[k], (double)lo[k]);  // exact
-    } else {
-      // binary64 sum in ascending point index (the grouped order; rare: large
-      // dynamic range)
-#pragma unroll
-      for (int k = 0; k < 9; ++k) sum[k] = 0.0;
-      for (uint32_t a = 0; a < c; ++a) {
-        const int64_t d = (int64_t)o + a;
-#pragma unroll
-        for (int k = 0; k < 3; ++k) sum[k] = __dadd_rn(sum[k], (double)gpts[3 * d + k]);
-#pragma unroll
-        for (int k = 0; k < 6; ++k) sum[3 + k] = __dadd_rn(sum[3 + k], (double)gcovs[6 * d + k]);
-      }
-    }
     const double N = (double)c;
     const double y = __drcp_rn(N);
 #pragma unroll
     for (int k = 0; k < 9; ++k)
-      if (need64 & (1u << k)) q[k] = __double2float_rn(div_rn(sum[k], N, y));
+      if (need64 & (1u << k)) {
+        const double sum = exact ? __dadd_rn((double)hi[k], (double)lo[k])  // exact
+                                 : get_sum64(hi[k], lo[k]);
+        q[k] = __double2float_rn(div_rn(sum, N, y));
+      }
   }
   recs[3 * v + 0] = make_float4(q[0], q[1], q[2], __uint_as_float(c));
   recs[3 * v + 1] = make_float4(q[3], q[4], q[5], q[6]);
@@ -464,8 +486,10 @@ __global__ void __launch_bounds__(kFinThreads) finalize_kernel(
 #pragma unroll
       for (int k = 0; k < 9; ++k) hi[k] = lo[k] = 0.0f;
       bool exact = true;
-      sum_entries(gpts, gcovs, o, c, 0u, 1u, hi, lo, exact);
-      write_record(v, o, c, hi, lo, exact, gpts, gcovs, recs, q);
+      uint32_t low = 0u;
+      sum_entries<false>(gpts, gcovs, o, c, 0u, 1u, hi, lo, exact, low);
+      if (!exact) sum_entries64(gpts, gcovs, o, c, hi, lo);
+      write_record(v, c, hi, lo, exact, recs, q);
       // the voxel's map (ranks and voxel ids of a map share its range
       // [vbase[m], vbase[m + 1])): a CTA's ranks rarely span two maps
       int m = seg_map[0];
@@ -495,13 +519,54 @@ __device__ __forceinline__ void add_lane(float* hi, float* lo, bool& exact, int 
   }
 }
 
+// The sums of the nine components of list entries o .. o + c - 1 in ascending point index,
+// one by each of a warp's first lanes: as sum_entries, or (words of) the binary64 sums where
+// one of those is not exact.  Returns whether they all are.
+__device__ __forceinline__ bool sum_components(const float* gpts, const float* gcovs, int lane,
+                                               uint32_t o, uint32_t c, float& hi, float& lo) {
+  const float* const f = lane < 3 ? gpts + 3 * (int64_t)o + lane : gcovs + 6 * (int64_t)o + (lane - 3);
+  const int step = lane < 3 ? 3 : 6;
+  const uint32_t n = lane < 9 ? c : 0u;
+  bool exact = true;
+#pragma unroll 4
+  for (uint32_t a = 0; a < n; ++a) {
+    float t, e, u, e2;
+    two_sum(hi, f[(int64_t)step * a], t, e);
+    two_sum(lo, e, u, e2);
+    exact = exact && e2 == 0.0f;
+    hi = t;
+    lo = u;
+  }
+  if (__all_sync(0xFFFFFFFFu, exact)) return true;
+  double sum = 0.0;
+#pragma unroll 4
+  for (uint32_t a = 0; a < n; ++a) sum = __dadd_rn(sum, (double)f[(int64_t)step * a]);
+  put_sum64(sum, hi, lo);
+  return false;
+}
+
+// Whether the order of a list's exact sums cannot matter (hi: the sums, low: the least
+// off-diagonal magnitude): the partial sums, below the largest diagonal sum (covariances are
+// positive semi-definite), are multiples of the last bit of the smallest and at most 2^53 of
+// them, so that the sums in ascending point index are exact too.  (Coordinates, which have
+// one sign in a voxel, and diagonal entries do not cancel.)
+__device__ __forceinline__ bool any_order(const float* hi, uint32_t low) {
+  const float top = fmaxf(fabsf(hi[3]), fmaxf(fabsf(hi[6]), fabsf(hi[8])));
+  const int e = (int)(__float_as_uint(top) >> 23) + 1;
+  return low == 0xFFFFFFFFu || (e < 255 && e - max((int)((low + 1u) >> 24), 1) <= 30);
+}
+
 // The same for long lists: R consecutive ranks per CTA, 128 / R threads per voxel, R
 // the power of two that makes about 512 points per CTA.  The lists are not sorted
 // first: a point's position in the grouped cloud is the number of smaller indices in
 // its list, counted by the thread that copies it.  A voxel's threads sum its points
 // (exact partial sums, joined exactly); a list longer than 64 points per thread is
-// summed by the whole warp.  A segment longer than the staging buffer (a voxel of
-// thousands of points) is sorted in place by one thread per voxel, as above.
+// summed by the whole warp.  Where the order of the points may matter, or the sums are not
+// exact, nine lanes sum the list once more in ascending point index, a component each (a
+// list of 160 points that one lane summed in binary64 took 100 us; rebuild of ten maps of
+// 20,000 points at 100 per voxel, one such list 185 -> 99 us, none 86).  A segment longer
+// than the staging buffer (a voxel of thousands of points) is sorted in place by one thread
+// per voxel, as above.
 // Bounded by the latency of the chain offsets - indices - gather - sums on few CTAs.
 // This kernel / the one above (points per voxel on average): ten maps of 20,000
 // points 19 / 18 us (2.0), 20 / 28 (5.7), 19 / 55 (11), 21 / 148 (23), 49 / 1554 (91);
@@ -587,20 +652,27 @@ __global__ void __launch_bounds__(kFinThreads, 6) finalize_long_kernel(
 #pragma unroll
     for (int k = 0; k < 9; ++k) hi[k] = lo[k] = 0.0f;
     bool exact = true;
+    uint32_t low = 0xFFFFFFFFu;
     const bool by_warp = c > kFinSerial * (uint32_t)per;
-    if (!by_warp) sum_entries(gpts, gcovs, o, c, part, per, hi, lo, exact);
-    for (int d = 1; d < per; d <<= 1) add_lane(hi, lo, exact, d);
+    if (!by_warp) sum_entries<true>(gpts, gcovs, o, c, part, per, hi, lo, exact, low);
+    for (int d = 1; d < per; d <<= 1) {
+      add_lane(hi, lo, exact, d);
+      low = min(low, __shfl_xor_sync(0xFFFFFFFFu, low, d));
+    }
     for (uint32_t todo = __ballot_sync(0xFFFFFFFFu, mine && by_warp); todo; todo &= todo - 1u) {
       const int b = __ffs(todo) - 1;  // the whole warp sums the list of lane b
       const uint32_t ob = __shfl_sync(0xFFFFFFFFu, o, b), cb = __shfl_sync(0xFFFFFFFFu, c, b);
       float h[9], l[9];
       bool ex = true;
+      uint32_t lw = 0xFFFFFFFFu;
 #pragma unroll
       for (int k = 0; k < 9; ++k) h[k] = l[k] = 0.0f;
-      sum_entries(gpts, gcovs, ob, cb, lane, 32u, h, l, ex);
+      sum_entries<true>(gpts, gcovs, ob, cb, lane, 32u, h, l, ex, lw);
 #pragma unroll 1
       for (int d = 1; d < 32; d <<= 1) add_lane(h, l, ex, d);
+      lw = __reduce_min_sync(0xFFFFFFFFu, lw);
       if (lane == b) {
+        low = lw;
 #pragma unroll
         for (int k = 0; k < 9; ++k) {
           hi[k] = h[k];
@@ -609,8 +681,24 @@ __global__ void __launch_bounds__(kFinThreads, 6) finalize_long_kernel(
         exact = ex;
       }
     }
+    const bool again = mine && (!exact || ((per > 1 || by_warp) && !any_order(hi, low)));
+    for (uint32_t todo = __ballot_sync(0xFFFFFFFFu, again); todo; todo &= todo - 1u) {
+      const int b = __ffs(todo) - 1;  // the list of lane b in ascending index, by nine lanes
+      const uint32_t ob = __shfl_sync(0xFFFFFFFFu, o, b), cb = __shfl_sync(0xFFFFFFFFu, c, b);
+      float h = 0.0f, l = 0.0f;
+      const bool ex = sum_components(gpts, gcovs, lane, ob, cb, h, l);
+#pragma unroll
+      for (int k = 0; k < 9; ++k) {
+        const float hk = __shfl_sync(0xFFFFFFFFu, h, k), lk = __shfl_sync(0xFFFFFFFFu, l, k);
+        if (lane == b) {
+          hi[k] = hk;
+          lo[k] = lk;
+        }
+      }
+      if (lane == b) exact = ex;
+    }
     if (mine) {
-      write_record(v, o, c, hi, lo, exact, gpts, gcovs, recs, q);
+      write_record(v, c, hi, lo, exact, recs, q);
       insert_lookup(v, vkeys[v], c, q, map_of_rank(vbase, n_maps, r), slot_base, vmask, max_probe,
                     vslots, lslot_of, status);
     }
