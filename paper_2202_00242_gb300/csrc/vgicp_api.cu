@@ -135,6 +135,7 @@ int create_set(const int64_t* offsets, int32_t n_maps, double resolution,
   }
   s->n_chunks = (int32_t)chunks.size();
   const size_t o_chunks = take(sizeof(int2) * chunks.size());
+  const size_t o_chunk_points = take(sizeof(uint32_t) * chunks.size());
   const size_t o_goff = take(sizeof(uint32_t) * n);
   const size_t o_gpts = take(sizeof(float) * 3 * n);
   const size_t o_gcovs = take(sizeof(float) * 6 * n);
@@ -170,6 +171,7 @@ int create_set(const int64_t* offsets, int32_t n_maps, double resolution,
   s->d_gpts = reinterpret_cast<float*>(b + o_gpts);
   s->d_goff = reinterpret_cast<uint32_t*>(b + o_goff);
   s->d_chunks = reinterpret_cast<int2*>(b + o_chunks);
+  s->d_chunk_points = reinterpret_cast<uint32_t*>(b + o_chunk_points);
   s->d_gcovs = reinterpret_cast<float*>(b + o_gcovs);
   s->d_scan_tmp = reinterpret_cast<uint32_t*>(b + o_scan);
   cudaGetDevice(&s->device);

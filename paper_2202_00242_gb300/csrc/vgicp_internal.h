@@ -79,6 +79,7 @@ struct MapSet {
   float* d_gcovs = nullptr;       // n_total x 6   Morton order (within chunks of a map)
   uint32_t* d_goff = nullptr;     // n_total: grouped offset of each Morton rank
   int2* d_chunks = nullptr;       // (map, chunk) pairs for the Morton sort
+  uint32_t* d_chunk_points = nullptr;  // n_chunks: points of each chunk's voxels
   int32_t n_chunks = 0;
   uint32_t* d_scan_tmp = nullptr; // scan block sums
   uint32_t* d_num_voxels = nullptr;  // 1 (total V)
