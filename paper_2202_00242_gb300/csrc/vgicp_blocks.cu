@@ -30,6 +30,10 @@ __device__ __forceinline__ void leave_to_probes(const BlockMap& M) {
   M.state[0] = 1u;
   *M.any = 1u;
 }
+// Whether the map has been left to the probes (by this kernel perhaps, and meanwhile).
+__device__ __forceinline__ bool is_left(const BlockMap& M) {
+  return *(const volatile uint32_t*)M.state != 0u;
+}
 
 __global__ void __launch_bounds__(kThreads) block_insert_kernel(const BlockMap* __restrict__ maps) {
   const BlockMap M = maps[blockIdx.y];
@@ -38,6 +42,8 @@ __global__ void __launch_bounds__(kThreads) block_insert_kernel(const BlockMap* 
     if (blockIdx.x == 0 && threadIdx.x == 0) leave_to_probes(M);
     return;
   }
+  // a map of scattered voxels, a block or nearly one to each, fills its table early on
+  if (is_left(M)) return;
   const unsigned long long fm = (1ull << kKeyBits) - 1ull;
   for (uint32_t i = blockIdx.x * kThreads + threadIdx.x; i < V; i += gridDim.x * kThreads) {
     const unsigned long long k = M.vkeys[v0 + i];
@@ -56,6 +62,7 @@ __global__ void __launch_bounds__(kThreads) block_insert_kernel(const BlockMap* 
           if (cur == 0ull && atomicAdd(M.state + 2, 1u) >= M.mask / 4u * 3u) leave_to_probes(M);
           break;
         }
+        if ((p & 7) == 7 && is_left(M)) return;
         h = (h + 1) & M.mask;
       }
       if (found != kNoSlot)
@@ -70,6 +77,7 @@ __global__ void __launch_bounds__(kThreads) block_insert_kernel(const BlockMap* 
 
 __global__ void __launch_bounds__(kThreads) block_place_kernel(const BlockMap* __restrict__ maps) {
   const BlockMap M = maps[blockIdx.y];
+  if (is_left(M)) return;
   __shared__ uint32_t warp_sum[kThreads / 32];
   __shared__ uint32_t base;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -102,8 +110,8 @@ __global__ void __launch_bounds__(kThreads) block_place_kernel(const BlockMap* _
 
 __global__ void __launch_bounds__(kThreads) block_fill_kernel(const BlockMap* __restrict__ maps) {
   const BlockMap M = maps[blockIdx.y];
+  if (is_left(M)) return;
   const uint32_t v0 = M.vbase[0], V = M.vbase[1] - v0;
-  if (V > M.rec_cap) return;
   const unsigned long long fm = (1ull << kKeyBits) - 1ull;
   for (uint32_t i = blockIdx.x * kThreads + threadIdx.x; i < V; i += gridDim.x * kThreads) {
     const uint32_t s = M.block_of[i];
