@@ -148,6 +148,20 @@ __global__ void copy_results_kernel(double* __restrict__ out, int64_t* __restric
   }
 }
 
+// Whether a kernel on the plan's device may store 8-byte words at p, or p is null: device
+// memory of that device, aligned.  Anything else is left to a copy, which takes it or
+// reports it.
+bool storable(const void* p, int device) {
+  if (!p) return true;
+  if ((uintptr_t)p & 7u) return false;
+  cudaPointerAttributes a;
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return a.type == cudaMemoryTypeDevice && a.device == device;
+}
+
 // The poses go to the device through a kernel that reads the pinned staging
 // buffer, not through a copy engine: a host-to-device copy queued there would
 // wait behind whatever large upload the caller has in flight (for instance the
@@ -459,7 +473,14 @@ int vgicp_plan_execute(vgicp_plan* P, const double* poses, double* out, int64_t*
   VGICP_CUDA_TRY(cudaGraphLaunch(P->exec, st));
   count_launches(2);  // linearize + reduce
   if (kernel_stop) VGICP_CUDA_TRY(cudaEventRecord(static_cast<cudaEvent_t>(kernel_stop), st));
-  if (out || inliers) {
+  if (!storable(out, P->device) || !storable(inliers, P->device)) {
+    if (out)
+      VGICP_CUDA_TRY(cudaMemcpyAsync(out, P->d_out, sizeof(double) * 43 * P->n_pairs,
+                                     cudaMemcpyDeviceToDevice, st));
+    if (inliers)
+      VGICP_CUDA_TRY(cudaMemcpyAsync(inliers, P->d_inl, sizeof(int64_t) * P->n_pairs,
+                                     cudaMemcpyDeviceToDevice, st));
+  } else if (out || inliers) {
     const int64_t n_out = 43 * (int64_t)P->n_pairs, n = n_out + P->n_pairs;
     copy_results_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(out, inliers, P->d_out,
                                                                     P->d_inl, n_out, P->n_pairs);
