@@ -64,6 +64,12 @@ int vgicp_version(void);
  * (all threads, all devices); for accounting in benchmarks. */
 int64_t vgicp_launch_count(void);
 
+/* Gives back the device memory that the library keeps for the scratch of its
+ * calls (up to 512 MB per device, all devices), as far as no call is using it; the
+ * next calls take theirs anew.  Happens by itself when the last map or plan is
+ * destroyed.  Scratch of calls still running stays until they have run. */
+int vgicp_release_scratch(void);
+
 /* Fault injection for tests of error handling (no counterpart in the paper):
  * the next `count` device allocations the library would make fail with
  * VGICP_ERR_OOM, without calling the allocator, exactly as a real out-of-memory

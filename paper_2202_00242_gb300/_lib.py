@@ -34,6 +34,7 @@ SIGNATURES = {
     "vgicp_last_error_string": (ctypes.c_char_p, []),
     "vgicp_version": (ctypes.c_int, []),
     "vgicp_launch_count": (i64, []),
+    "vgicp_release_scratch": (ctypes.c_int, []),
     "vgicp_test_fail_allocations": (ctypes.c_int, [i32]),
     "vgicp_test_expire_waits": (ctypes.c_int, [i32, i64]),
     "vgicp_build_voxelmap": (ctypes.c_int, [P, P, i64, f64, ctypes.POINTER(MapOpts), P,

@@ -503,6 +503,14 @@ def downsample(points: torch.Tensor, resolution: float, times: torch.Tensor | No
     return op[:V], (ot[:V] if ot is not None else None), oc[:V], oo
 
 
+def release_scratch():
+    """Give the device memory that the library keeps for its calls' scratch (up to 512 MB
+    per device) back.  It goes back by itself with the last map or plan; a program that
+    only downsamples or estimates covariances calls this when something else needs the
+    memory."""
+    check(_lib.load().vgicp_release_scratch())
+
+
 def estimate_covariances(points: torch.Tensor, offsets=None, k: int = 10, eps: float = 1e-3,
                          cell: float = 0.0, neighbours: bool = False, stream=None):
     """Regularised k-nearest-neighbour covariances (Sec. III-C) of each point of

@@ -237,8 +237,10 @@ std::atomic<int32_t> g_fail_allocs{0};
 // time: one factor of 8,192 points took 251 us waited for, 35 us among others.  The
 // library's pool keeps up to kScratchKept bytes between calls; what exceeds it goes
 // back at a synchronization, and all of it when the process's last map or plan is
-// destroyed or when an allocation of the library fails.  The allocator itself
-// orders reuse between streams and is safe from several threads.
+// destroyed, when an allocation of the library fails, or when the program asks
+// (vgicp_release_scratch: one that only downsamples or estimates covariances has no map
+// whose end could be the occasion).  The allocator itself orders reuse between streams
+// and is safe from several threads.
 constexpr uint64_t kScratchKept = 512ull << 20;
 std::mutex g_pool_mutex;
 cudaMemPool_t g_pool[kMaxDevices] = {nullptr};
@@ -269,11 +271,16 @@ static cudaMemPool_t scratch_pool(bool create) {
   return g_pool[dev];
 }
 
-void count_owners(int n) {
-  if (g_owners.fetch_add(n, std::memory_order_relaxed) + n > 0 || n > 0) return;
+// What no call is using goes back to the device.
+static void trim_pools() {
   std::lock_guard<std::mutex> lock(g_pool_mutex);
   for (cudaMemPool_t pool : g_pool)
     if (pool && cudaMemPoolTrimTo(pool, 0) != cudaSuccess) cudaGetLastError();
+}
+
+void count_owners(int n) {
+  if (g_owners.fetch_add(n, std::memory_order_relaxed) + n > 0 || n > 0) return;
+  trim_pools();
 }
 
 cudaError_t device_malloc(void** p, size_t bytes, cudaStream_t st, bool stream_ordered) {
@@ -331,6 +338,12 @@ const char* vgicp_last_error_string(void) { return g_error.c_str(); }
 int vgicp_version(void) { return 10000; }
 
 int64_t vgicp_launch_count(void) { return g_launches.load(std::memory_order_relaxed); }
+
+int vgicp_release_scratch(void) {
+  g_error.clear();
+  trim_pools();
+  return VGICP_OK;
+}
 
 int vgicp_test_fail_allocations(int32_t count) {
   if (count < 0) return set_error(VGICP_ERR_INVALID_ARG, "negative count");
