@@ -252,7 +252,8 @@ int vgicp_linearize_batched(vgicp_map* const* maps, int32_t n_maps, const vgicp_
  *           W = (C' + R C R^T)^-1 with the rotation, -u^T (dM/domega_i) u with
  *           u = W d, and err.
  * out: device n_pairs x 7 doubles (gradient 6, err 1); inliers as before.
- * Runs the one-point-per-thread kernel. */
+ * The results are those of the one-point-per-thread kernel (variant 1), whatever
+ * opts->variant says; few work items go to kernels that sum them alike. */
 int vgicp_evaluate_batched(vgicp_map* const* maps, int32_t n_maps, const vgicp_cloud* sources,
                            int32_t n_sources, const int32_t* pairs, int64_t n_pairs,
                            const double* poses, int32_t mode, double* out, int64_t* inliers,
@@ -390,7 +391,7 @@ int vgicp_plan_autotune(vgicp_plan* plan, const double* poses, vgicp_stream_t st
 
 /* Linearize all factors at poses (host, n_pairs x 16 doubles, read during the
  * call).  out: device n_pairs x 43, inliers: device n_pairs (either may be NULL;
- * results are copied there after the graph).  kernel_start/kernel_stop:
+ * results are copied there after the graph, fastest to 8-byte aligned buffers).  kernel_start/kernel_stop:
  * optional cudaEvent_t recorded on the stream around the graph launch (status
  * reset, linearize kernel, per-pair reduction).  The first call captures the
  * graph. */
@@ -399,9 +400,10 @@ int vgicp_plan_execute(vgicp_plan* plan, const double* poses, double* out, int64
 
 /* Differentiable evaluation (Sec. III-A: the matching cost as a function of the
  * pose, differentiated for a gradient-based optimizer).  Every factor p is
- * evaluated at T_p = T0_p Exp(xi_p), composed on the device in binary64, with
- * the one-point-per-thread kernel and the plan's work list; nothing is copied
- * to or from the host and the call does not synchronize.
+ * evaluated at T_p = T0_p Exp(xi_p), composed on the device in binary64, over
+ * the plan's work list, with the results of the one-point-per-thread kernel
+ * (variant 1); nothing is copied to or from the host and the call does not
+ * synchronize.
  *   base_poses: device, n_pairs x 16 doubles (row-major T0_p, finite rigid).
  *   xi:         device, n_pairs x 6 doubles ([omega; v]), or NULL for xi = 0.
  *   mode 1: err only; 2: gradient with W held, 2 J^T W d; 3: exact gradient
