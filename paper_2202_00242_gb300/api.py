@@ -638,9 +638,10 @@ def linearize_admitted(points_host, covs_host, offsets, pairs, poses, resolution
     (rebuilt in place); the last set is released at the end.
     ``points_host`` / ``covs_host``: numpy arrays or CPU tensors (pinned tensors
     upload at full speed).  ``budget`` counts the maps and clouds of a batch; a call's
-    scratch (partial sums, with 27 neighbours occupancy blocks of about 100 bytes a voxel,
-    which are left out where they cannot be had) comes on top.  Returns (out (P, 43) float64 host, inliers (P,) host,
-    n_batches).  ``kernel_events``: optional list; each batch appends the
+    scratch (partial sums, with 27 neighbours occupancy blocks of about 100 bytes a
+    voxel, which are left out where they cannot be had) comes on top.  Returns
+    (out (P, 43) float64 host, inliers (P,) host, n_batches).  ``kernel_events``:
+    optional list; each batch appends the
     (start, stop) torch.cuda.Event pair recorded around its linearize kernel."""
     off = np.asarray(offsets, dtype=np.int64)
     pairs = np.ascontiguousarray(np.asarray(pairs, dtype=np.int32).reshape(-1, 2))

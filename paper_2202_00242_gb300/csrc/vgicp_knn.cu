@@ -19,8 +19,8 @@
 //             (within 2^-21 of the binary64 value); values closer than that bound
 //             allows are decided in binary64.
 //   covariance  mean of the k neighbours and their scatter about it, in float32
-//             relative to the query point, the eigenvector v of the smallest eigenvalue by cyclic
-//             Jacobi (float32, on the trace-normalised matrix), and
+//             relative to the query point, the eigenvector v of the smallest
+//             eigenvalue by cyclic Jacobi (float32, on the trace-normalised matrix), and
 //             C = V diag(1, 1, eps) V^T = I - (1 - eps) v v^T.
 #include <cuda_runtime.h>
 
