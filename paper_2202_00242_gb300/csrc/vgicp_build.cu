@@ -16,9 +16,11 @@
 //             its count, key and, in the slot, its id
 //             (and per map: lookup-table capacity from the voxel count)
 //   sort      per map chunk: the voxels in Morton order of their keys (rank), and
-//             the offsets of their point lists, in rank order and by voxel
+//             the offsets of their point lists, in rank order and by voxel (for
+//             maps of many chunks after a kernel that counts the chunks' points)
 //   scatter   per point: append its index to its voxel's list; the voxel's
-//             last point empties its build-table slot
+//             last point empties its build-table slot (a point without a voxel is
+//             marked behind its map's last list)
 //   finalize  per voxel, in rank order: sort its list, sum means and
 //             covariances (exactly, else in binary64 in ascending point index),
 //             divide by N, round to float32; copy the points into the voxel-
@@ -396,9 +398,9 @@ __device__ __forceinline__ void write_record(uint32_t v, uint32_t c, float* hi, 
   recs[3 * v + 2] = make_float4(q[7], q[8], 0.0f, 0.0f);
 }
 
-// One read of a word that other CTAs may be setting, whose value then stays.  (Rebuild of
-// 500 maps of 50,000 points: 3,091 us so, 3,101 with a relaxed and 3,110 with a volatile
-// load, which the kernel's other loads wait for.)
+// One read of a word that other CTAs may be setting, whose value then stays.  (A relaxed
+// load, which the kernel's other loads wait for, takes the rebuild of 500 maps of 50,000
+// points 10 us more, of 3.1 ms, a volatile one 20.)
 __device__ __forceinline__ int32_t read_once(const int32_t* p) {
   int32_t v;
   asm("ld.global.b32 %0, [%1];" : "=r"(v) : "l"(p));
