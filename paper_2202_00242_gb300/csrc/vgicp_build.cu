@@ -39,6 +39,7 @@
 #include "vgicp_device.cuh"
 #include "vgicp_internal.h"
 #include "vgicp_mean.h"
+#include "vgicp_sort.cuh"
 
 namespace vgicp {
 namespace {
@@ -273,18 +274,6 @@ __device__ __forceinline__ void insert_lookup(uint32_t v, unsigned long long key
 constexpr int kFinThreads = 128;
 constexpr int kFinStage = 3072;  // indices staged per CTA
 
-__device__ __forceinline__ void insertion_sort(uint32_t* L, uint32_t c) {
-  for (uint32_t a = 1; a < c; ++a) {
-    const uint32_t x = L[a];
-    int b = (int)a - 1;
-    while (b >= 0 && L[b] > x) {
-      L[b + 1] = L[b];
-      --b;
-    }
-    L[b + 1] = x;
-  }
-}
-
 // Map of rank (or voxel id) r: the last m with vbase[m] <= r.
 __device__ __forceinline__ int map_of_rank(const uint32_t* __restrict__ vbase, int32_t n_maps,
                                            int64_t r) {
@@ -461,7 +450,7 @@ __global__ void __launch_bounds__(kFinThreads) finalize_kernel(
       __syncthreads();
       if (mine) insertion_sort(stage + (o - seg0), c);
     } else if (mine) {
-      insertion_sort(plist + o, c);
+      sort_list(plist + o, c);
     }
     __syncthreads();
     // 2. gather into the grouped cloud
@@ -617,7 +606,7 @@ __global__ void __launch_bounds__(kFinThreads, 6) finalize_long_kernel(
       for (uint32_t i = threadIdx.x; i < len; i += kFinThreads) stage[i] = plist[seg0 + i];
       if (mine) list_at[r - r0] = o - seg0;
     } else if (mine) {
-      insertion_sort(plist + o, c);
+      sort_list(plist + o, c);
     }
     __syncthreads();
     for (uint32_t i = threadIdx.x; i < len; i += kFinThreads) {

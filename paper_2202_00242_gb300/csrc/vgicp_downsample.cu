@@ -38,6 +38,7 @@
 #include "vgicp.h"
 #include "vgicp_device.cuh"
 #include "vgicp_internal.h"
+#include "vgicp_sort.cuh"
 
 namespace vgicp {
 namespace {
@@ -447,15 +448,7 @@ __global__ void __launch_bounds__(kThreads) ds_finalize_kernel(
           if (a < (int)c) add_64(e[a]);
     } else {
       uint32_t* L = list + at;
-      for (uint32_t a = 1; a < c; ++a) {
-        const uint32_t x = L[a];
-        int b = (int)a - 1;
-        while (b >= 0 && L[b] > x) {
-          L[b + 1] = L[b];
-          --b;
-        }
-        L[b + 1] = x;
-      }
+      sort_list(L, c);
       for (uint32_t a = 0; a < c; ++a) add_exact(L[a]);
       if (!exact)
         for (uint32_t a = 0; a < c; ++a) add_64(L[a]);
