@@ -549,6 +549,42 @@ __device__ __forceinline__ bool any_order(const float* hi, uint32_t low) {
   return low == 0xFFFFFFFFu || (e < 255 && e - max((int)((low + 1u) >> 24), 1) <= 30);
 }
 
+// What any_order leaves open, by component, `per` lanes to a list: whether the entries off
+// the diagonal are multiples of the last bit of their component's smallest and their
+// partial sums, at most c times the largest, below 2^53 of those.  (Off-diagonal entries
+// that are all tiny, of planes along an axis, stay open above.)
+__device__ __forceinline__ bool off_diagonals_fit(const float* gcovs, uint32_t o, uint32_t c,
+                                                  int part, int per) {
+  uint32_t low[3], top[3];  // bits less one (zeros last), bits
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    low[k] = 0xFFFFFFFFu;
+    top[k] = 0u;
+  }
+  for (uint32_t a = part; a < c; a += per) {
+    const float* const f = gcovs + 6 * ((int64_t)o + a);
+    const float v[3] = {f[1], f[2], f[4]};
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const uint32_t b = __float_as_uint(v[k]) & 0x7FFFFFFFu;
+      low[k] = min(low[k], b - 1u);
+      top[k] = max(top[k], b);
+    }
+  }
+  bool fits = true;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    for (int d = 1; d < per; d <<= 1) {
+      low[k] = min(low[k], __shfl_xor_sync(0xFFFFFFFFu, low[k], d));
+      top[k] = max(top[k], __shfl_xor_sync(0xFFFFFFFFu, top[k], d));
+    }
+    const int e_top = max((int)(top[k] >> 23), 1), e_low = max((int)((low[k] + 1u) >> 23), 1);
+    fits = fits && (top[k] == 0u ||
+                    (e_top < 255 && e_top - e_low + 32 - __clz((int)(c - 1u)) <= 29));
+  }
+  return fits;
+}
+
 // The same for long lists: R consecutive ranks per CTA, 128 / R threads per voxel, R
 // the power of two that makes about 512 points per CTA.  The lists are not sorted
 // first: a point's position in the grouped cloud is the number of smaller indices in
@@ -674,7 +710,13 @@ __global__ void __launch_bounds__(kFinThreads, 6) finalize_long_kernel(
         exact = ex;
       }
     }
-    const bool again = mine && (!exact || ((per > 1 || by_warp) && !any_order(hi, low)));
+    bool open = mine && exact && (per > 1 || by_warp) && !any_order(hi, low);
+    if (__any_sync(0xFFFFFFFFu, open)) {  // by component, by the lists' threads
+      open = __shfl_sync(0xFFFFFFFFu, (int)open, lane & ~(per - 1)) != 0;
+      const bool fits = off_diagonals_fit(gcovs, o, open ? c : 0u, part, per);
+      open = open && !fits;
+    }
+    const bool again = mine && (!exact || open);
     for (uint32_t todo = __ballot_sync(0xFFFFFFFFu, again); todo; todo &= todo - 1u) {
       const int b = __ffs(todo) - 1;  // the list of lane b in ascending index, by nine lanes
       const uint32_t ob = __shfl_sync(0xFFFFFFFFu, o, b), cb = __shfl_sync(0xFFFFFFFFu, c, b);

@@ -58,3 +58,18 @@ def test_means_on_midpoints(dev, members, tiny):  # noqa: F811
     vm = api.VoxelMap.build(cu(pts), cu(covs), 1.0)
     vm.status()
     check_export(vm, pts, covs, 1.0)
+
+
+@pytest.mark.parametrize("members", [8, 24, 70, 200, 2100])
+@pytest.mark.parametrize("scale", [1e-6, 1e-9, 1e-20, 0.0])
+def test_entries_that_are_all_tiny(dev, members, scale):  # noqa: F811
+    """Planes along an axis: off-diagonal entries far below the diagonal ones, in one list in
+    three with a larger one among them."""
+    pts, v, rng = _voxels(members, 40 if members > 1000 else 300, members)
+    off = rng.normal(size=(len(v), 3)) * scale
+    off[::3 * members, 1] = 0.25
+    covs = np.column_stack([1 + rng.random(len(v)), off[:, 0], off[:, 1], 1 + rng.random(len(v)),
+                            off[:, 2], np.full(len(v), 1.0)]).astype(np.float32)
+    vm = api.VoxelMap.build(cu(pts), cu(covs), 1.0)
+    vm.status()
+    check_export(vm, pts, covs, 1.0)
